@@ -25,7 +25,8 @@ struct ProjNum {
   static __device__ __forceinline__ T in(TS x) { return (T)x; }
   template <typename TS>
   static __device__ __forceinline__ TS out(T x) { return (TS)x; }
-  static __device__ __forceinline__ T shfl1(T v) { return __shfl_xor_sync(0xffffffffu, v, 1); }
+  static __device__ __forceinline__ T shfl_xor(T v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+  static __device__ __forceinline__ T shfl1(T v) { return shfl_xor(v, 1); }
 };
 template <>
 struct ProjNum<ff2> {
@@ -34,9 +35,10 @@ struct ProjNum<ff2> {
   static __device__ __forceinline__ ff2 in(ff2 x) { return x; }
   template <typename TS>
   static __device__ __forceinline__ TS out(ff2 x) { return ff_to_double(x); }
-  static __device__ __forceinline__ ff2 shfl1(ff2 v) {
-    return ff_make(__shfl_xor_sync(0xffffffffu, v.hi, 1), __shfl_xor_sync(0xffffffffu, v.lo, 1));
+  static __device__ __forceinline__ ff2 shfl_xor(ff2 v, int o) {
+    return ff_make(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
   }
+  static __device__ __forceinline__ ff2 shfl1(ff2 v) { return shfl_xor(v, 1); }
 };
 
 constexpr int kProjWarps = 8;
@@ -157,8 +159,9 @@ __host__ __device__ constexpr int pair_fstride() {
 // P[pr][b][col] = sum_node conj(F[pr][b][node]) x(d(node), col), x scaled by
 // D^{-1/2} when dscale is given.  Each thread owns V = 16 / sizeof(TS)
 // adjacent columns (one 16-byte load per row; for complex data the re/im
-// partner is in the same thread); cg column groups per CTA, the 256 / cg row
-// slices of a CTA reduced in shared memory in slice order.  MAXP >= n_proj.
+// partner is in the same thread); cg (a power of two) column groups per CTA, the
+// 256 / cg row slices of a CTA reduced within each warp by shuffles (cg < 32) and
+// then in shared memory in slice order.  MAXP >= n_proj.
 template <typename T, typename TS, typename TF, bool CPLX, int MAXP>
 __global__ void __launch_bounds__(kPairThreads)
 fe_proj_pair_kernel(const TS* __restrict__ Xg, int64_t ld, int ncols, const int* __restrict__ cell_dofs,
@@ -252,6 +255,13 @@ fe_proj_pair_kernel(const TS* __restrict__ Xg, int64_t ld, int ncols, const int*
       }
     }
   }
+  // fewer than 32 groups: the warp's row slices, in a fixed tree
+  for (int o = 16; o >= cg; o >>= 1)
+#pragma unroll
+    for (int b = 0; b < MAXP; ++b)
+      if (b < n_proj)
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[b][v] = acc[b][v] + N::shfl_xor(acc[b][v], o);
   if (rs == 1) {
 #pragma unroll
     for (int b = 0; b < MAXP; ++b)
@@ -262,16 +272,18 @@ fe_proj_pair_kernel(const TS* __restrict__ Xg, int64_t ld, int ncols, const int*
     return;
   }
   const int cols = cg * V;   // columns of this CTA
+  const int ns = cg < 32 ? kPairThreads / 32 : rs, row = cg < 32 ? threadIdx.x / 32 : sl;   // partial sums left
+  if (cg >= 32 || (threadIdx.x & 31) < cg)
 #pragma unroll
-  for (int b = 0; b < MAXP; ++b)
-    if (b < n_proj)
+    for (int b = 0; b < MAXP; ++b)
+      if (b < n_proj)
 #pragma unroll
-      for (int v = 0; v < V; ++v) red[((size_t)sl * n_proj + b) * cols + lc * V + v] = acc[b][v];
+        for (int v = 0; v < V; ++v) red[((size_t)row * n_proj + b) * cols + lc * V + v] = acc[b][v];
   __syncthreads();
   for (int idx = threadIdx.x; idx < n_proj * cols; idx += kPairThreads) {
     const int b = idx / cols, c = idx % cols;
     T v = red[(size_t)b * cols + c];
-    for (int k = 1; k < rs; ++k) v = v + red[((size_t)k * n_proj + b) * cols + c];
+    for (int k = 1; k < ns; ++k) v = v + red[((size_t)k * n_proj + b) * cols + c];
     const int cc = blockIdx.y * cols + c;
     if (cc < ncols) part[((int64_t)pr * n_proj + b) * ld + cc] = N::template out<TS>(v);
   }
@@ -289,17 +301,32 @@ __global__ void fe_proj_sum_kernel(const TS* __restrict__ part, const TS* __rest
     const int64_t ab = idx / ncols;
     const int a = (int)(ab / n_proj), b = (int)(ab % n_proj);
     TS s = TS(0);
-    for (int pr = atom_pair_ptr[a]; pr < atom_pair_ptr[a + 1]; ++pr) s += part[((int64_t)pr * n_proj + b) * ld + col];
+    // 16 loads in flight (about a hundred pairs an atom; one after the other they cost the L2's latency each)
+    constexpr int U = 16;
+    int pr = atom_pair_ptr[a];
+    const int pe = atom_pair_ptr[a + 1];
+    const TS* src = part + ((int64_t)pr * n_proj + b) * ld + col;
+    const int64_t step = (int64_t)n_proj * ld;
+    for (; pr + U <= pe; pr += U, src += U * step) {
+      TS x[U];
+#pragma unroll
+      for (int k = 0; k < U; ++k) x[k] = src[k * step];
+#pragma unroll
+      for (int k = 0; k < U; ++k) s += x[k];
+    }
+    for (; pr < pe; ++pr, src += step) s += *src;
     Q[ab * ld + col] = s * h[ab];
   }
 }
 
 // Column groups (of 16 / sizeof(TS) columns) per CTA of the pair kernel: the
-// smallest multiple of 32 covering the columns, at most 256.
+// smallest power of two covering the columns, at most 256.  With fewer groups
+// than lanes the lanes of a warp take different rows (one column in pairs of
+// floats, 782 pairs at p = 8: 413 us when a group of columns filled a warp).
 template <typename TS>
 static int pair_groups(int ncols) {
   const int groups = (ncols + (16 / (int)sizeof(TS)) - 1) / (16 / (int)sizeof(TS));
-  int cg = 32;
+  int cg = 1;
   while (cg < 256 && cg < groups) cg *= 2;
   return cg;
 }
@@ -308,10 +335,10 @@ template <typename T, typename TS, typename TF, bool CPLX, int MAXP>
 static cudaError_t launch_pair_p(const ProjParams<TS>& prm, const TF* F, int n_atoms, cudaStream_t s) {
   constexpr int V = 16 / (int)sizeof(TS);
   const int cg = pair_groups<TS>(prm.ncols);
-  const int rs = kPairThreads / cg;
+  const int rs = kPairThreads / cg;   // row slices
   constexpr int PB = pair_fstride<TF, CPLX, MAXP>();
   const size_t head = ((size_t)prm.np3 * PB * sizeof(TF) + (size_t)prm.np3 * sizeof(int) + 15) & ~(size_t)15;
-  const size_t smem = head + (rs > 1 ? (size_t)rs * prm.n_proj * cg * V * sizeof(T) : 0);
+  const size_t smem = head + (rs > 1 ? (size_t)std::min(rs, cg < 32 ? kPairThreads / 32 : rs) * prm.n_proj * cg * V * sizeof(T) : 0);
   if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
   cudaError_t err = cudaFuncSetAttribute(fe_proj_pair_kernel<T, TS, TF, CPLX, MAXP>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
