@@ -1,8 +1,9 @@
 """Build libfe_ks.so in-tree with nvcc for sm_103a (no CMake).
 
 The translation units compile in parallel: the C-ABI / setup, the host 1D
-tables, the nonlocal kernels, and one object per FE degree of the fused local
-kernel (and per quadrature order n_q = n_p, n_p + 2).  Objects go to ``_build/`` beside this file; the shared library to
+tables, the nonlocal kernels, and one object per FE degree (and per quadrature
+order n_q = n_p, n_p + 2) of the fused local kernels and of the default cell
+kernel.  Objects go to ``_build/`` beside this file; the shared library to
 ``libfe_ks.so``.  A rebuild happens only when a source is newer than the
 library.
 """
@@ -33,15 +34,16 @@ def _nvcc():
 
 def _units():
     units = []
-    for name in ("fe_ks_api.cu", "fe_ks_tables.cu", "fe_ks_nonlocal.cu", "fe_ks_probe.cu", "fe_ks_cheb.cu", "fe_ks_static.cu", "fe_ks_batched.cu", "fe_ks_gemm.cu", "fe_ks_ffgemm.cu", "fe_ks_tc.cu", "fe_ks_cm.cu", "fe_ks_rr.cu", "fe_ks_tcgram.cu", "fe_ks_tc5.cu"):
+    for name in ("fe_ks_api.cu", "fe_ks_tables.cu", "fe_ks_nonlocal.cu", "fe_ks_probe.cu", "fe_ks_cheb.cu", "fe_ks_static.cu", "fe_ks_batched.cu", "fe_ks_gemm.cu", "fe_ks_ffgemm.cu", "fe_ks_tc.cu", "fe_ks_cm.cu", "fe_ks_rr.cu", "fe_ks_tcgram.cu", "fe_ks_tc5.cu", "fe_ks_assemble.cu"):
         units.append((os.path.join(CSRC, name), os.path.join(BUILD, name + ".o"), []))
     for nt in BATCH_THREADS:
         units.append((os.path.join(CSRC, "fe_ks_batched_k.cu"),
                       os.path.join(BUILD, f"fe_ks_batched_k{nt}.o"), [f"-DFEKS_BNT={nt}"]))
     for p in DEGREES:
         for nqx in NQ_OFFSETS:
-            units.append((os.path.join(CSRC, "fe_ks_local_deg.cu"),
-                          os.path.join(BUILD, f"fe_ks_local_p{p}_q{nqx}.o"), [f"-DFEKS_P={p}", f"-DFEKS_NQX={nqx}"]))
+            for unit in ("local", "line"):
+                units.append((os.path.join(CSRC, f"fe_ks_{unit}_deg.cu"), os.path.join(BUILD, f"fe_ks_{unit}_p{p}_q{nqx}.o"),
+                              [f"-DFEKS_P={p}", f"-DFEKS_NQX={nqx}"]))
     return units
 
 

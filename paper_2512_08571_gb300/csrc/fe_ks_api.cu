@@ -132,6 +132,22 @@ static fe_ks_status upload(Ctx* c, T** dst, const T* src, size_t count) {
   return FE_KS_OK;
 }
 
+int tiles_per_unit(int64_t cells, int ntiles, int64_t slots, double start, int multiple) {
+  int best = ntiles;
+  double least = 1e300;
+  for (int upc = 1; upc <= std::min(ntiles, 64); ++upc) {
+    int run = (ntiles + upc - 1) / upc;
+    run = (run + multiple - 1) / multiple * multiple;
+    const int64_t units = cells * ((ntiles + run - 1) / run);
+    const double t = (double)((units + slots - 1) / slots) * (run + start);
+    if (t <= 1.01 * least) {   // among equals the smaller units: cells with projectors take longer
+      least = std::min(t, least);
+      best = run;
+    }
+  }
+  return best;
+}
+
 // Greedy colouring of the cells so that no two cells of a colour share a DoF
 // (their scatter-adds then never touch the same row of Y).  Cells are taken
 // in index order; each gets the smallest colour not used by a cell sharing
@@ -164,6 +180,11 @@ int greedy_colouring(int64_t E, int np3, int64_t m, const int* cell_dofs, int* c
   }
   return n_colours;
 }
+
+// Most device memory a context sets aside for the slots of the one-launch
+// assembly.  Larger applications go colour by colour, where a colour's cells
+// then fill the device several times over and the launches cost nothing.
+constexpr size_t kAsmBytes = (size_t)256 << 20;
 
 // ---- tile-configuration cache: fe_ks_tune's choice per (degree, n_q,
 // precision, columns, complex, device), reused by contexts of the same shape
@@ -295,8 +316,9 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
   c->m = prob->n_dofs;
   c->n_v_max = n_v_max;
   c->terms = terms_mask;
-  c->stream = static_cast<cudaStream_t>(cuda_stream);
+  c->stream = c->home_stream = static_cast<cudaStream_t>(cuda_stream);
   cudaGetDevice(&c->device);
+  cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device);
   const double* kp = prob->kpt;
   c->cplx = (prob->force_complex != 0) || kp[0] != 0.0 || kp[1] != 0.0 || kp[2] != 0.0;
   c->gga = (terms_mask & FE_KS_TERM_G) && prob->v_gga_q != nullptr;
@@ -335,10 +357,17 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
   std::vector<double> coef((size_t)E * ncoef * nq3, 0.0);
   const double k2h = 0.5 * (kp[0] * kp[0] + kp[1] * kp[1] + kp[2] * kp[2]);
   std::atomic<int64_t> bad_det(-1);
+  // axis-aligned box cells: J diagonal and constant over the cell (to well below FP32
+  // rounding), so the kinetic and Bloch coefficients are a scalar of the cell times
+  // the point's weight
+  std::vector<float> cell_coef((size_t)E * 8, 0.f);
+  std::atomic<int> boxes(1);
   parallel_for(E, [&](int64_t b, int64_t e_end) {
     for (int64_t e = b; e < e_end; ++e) {
       const double* V = prob->cell_vertices + 24 * e;
       double* cf = coef.data() + (size_t)e * ncoef * nq3;
+      double J0[3] = {0.0, 0.0, 0.0};
+      bool box = true;
       for (int q = 0; q < nq3; ++q) {
         const int qx = q % nq, qy = (q / nq) % nq, qz = q / (nq * nq);
         const double xi[3] = {xg[qx], xg[qy], xg[qz]};
@@ -349,6 +378,11 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
           bad_det.store(e);
           continue;
         }
+        if (q == 0)
+          for (int d = 0; d < 3; ++d) J0[d] = J[d][d];
+        const double tiny = 1e-10 * std::fmin(std::fabs(J0[0]), std::fmin(std::fabs(J0[1]), std::fabs(J0[2])));
+        for (int s = 0; s < 3; ++s)
+          for (int d = 0; d < 3; ++d) box = box && std::fabs(J[s][d] - (s == d ? J0[s] : 0.0)) <= tiny;
         const double wd = det * wg[qx] * wg[qy] * wg[qz];
         if (terms_mask & FE_KS_TERM_T) {
           double K[3][3];
@@ -369,6 +403,14 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
         if (c->cplx && (terms_mask & FE_KS_TERM_K)) {
           for (int s = 0; s < 3; ++s)
             cf[(10 + s) * nq3 + q] = (Ji[s][0] * kp[0] + Ji[s][1] * kp[1] + Ji[s][2] * kp[2]) * wd;
+        }
+      }
+      if (!box) boxes.store(0, std::memory_order_relaxed);
+      if (box) {
+        const double det = J0[0] * J0[1] * J0[2];
+        for (int s = 0; s < 3; ++s) {
+          if (terms_mask & FE_KS_TERM_T) cell_coef[e * 8 + s] = (float)(0.5 * det / (J0[s] * J0[s]));
+          if (c->cplx && (terms_mask & FE_KS_TERM_K)) cell_coef[e * 8 + 4 + s] = (float)(kp[s] * det / J0[s]);
         }
       }
     }
@@ -416,6 +458,35 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
     for (int64_t e = 0; e < E; ++e)
       if (colour[e] == col) colour_cells.push_back((int)e);
     c->colour_ptr[col + 1] = (int)colour_cells.size();
+  }
+
+  // ---- one-launch assembly: rows met by one cell go straight to Y; every other (cell, node)
+  //      gets a slot, the slots of a DoF consecutive in the order in which the colour launches
+  //      would add them (the same bits either way)
+  std::vector<int> asm_dst((size_t)E * np3), asm_dof, asm_ptr;
+  {
+    std::vector<int> cnt(m, 0);
+    for (int64_t i = 0; i < E * np3; ++i) ++cnt[prob->cell_dofs[i]];
+    int64_t slots = 0;
+    for (int64_t d = 0; d < m; ++d) {
+      if (cnt[d] < 2) {
+        cnt[d] = -1;
+        continue;
+      }
+      asm_dof.push_back((int)d);
+      asm_ptr.push_back((int)slots);
+      const int n = cnt[d];
+      cnt[d] = (int)slots;
+      slots += n;
+    }
+    asm_ptr.push_back((int)slots);
+    for (const int e : colour_cells)
+      for (int i = 0; i < np3; ++i) {
+        const int d = prob->cell_dofs[(int64_t)e * np3 + i];
+        asm_dst[(int64_t)e * np3 + i] = cnt[d] < 0 ? d : ~cnt[d]++;
+      }
+    c->n_shared = (int64_t)asm_dof.size();
+    c->n_wslots = slots;
   }
 
   // ---- nonlocal projector matrices F^(a,e)[b][node] (eq. Vnonloc), cell -> pair CSR
@@ -548,6 +619,19 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
       ok = ok && chk(upload(c, &c->tc5_cst16, cst.data(), cst.size()));
     }
   }
+  if (ok) {
+    // slots for as many columns as kAsmBytes holds (all of n_v_max where that is less)
+    const size_t full = (size_t)c->n_wslots * n_v_max * (c->cplx ? 2 : 1) * sizeof(double);
+    c->asm_bytes = std::min(full, kAsmBytes);
+    ok = chk(upload(c, &c->asm_dst, asm_dst.data(), asm_dst.size())) &&
+         chk(upload(c, &c->asm_dof, asm_dof.data(), asm_dof.size())) &&
+         chk(upload(c, &c->asm_ptr, asm_ptr.data(), asm_ptr.size())) &&
+         chk(upload<char>(c, reinterpret_cast<char**>(&c->asm_W), nullptr, c->asm_bytes));
+  }
+  if (ok && boxes.load()) {
+    for (int q = 0; q < nq; ++q) c->gauss_w[q] = (float)wg[q];
+    ok = chk(upload(c, &c->cell_coef, cell_coef.data(), cell_coef.size()));
+  }
   if (ok && want_nl) {
     std::vector<double> hh(prob->h_coef, prob->h_coef + (size_t)prob->n_atoms * prob->n_proj);
     const size_t qn = (size_t)prob->n_atoms * prob->n_proj * n_v_max * (c->cplx ? 2 : 1);
@@ -661,6 +745,51 @@ fe_ks_status fe_ks_info(const fe_ks_ctx* ctx, int64_t* n_dofs, int64_t* n_cells,
 
 namespace feks {
 
+// Whether this application may go through the context's slots: the default kernel, slots
+// large enough, and nobody else in them.  An operator with projectors has per-context
+// scratch anyway (Q and its partials), so its applications are ordered by the caller; one
+// without has none, and may run on several streams at once: only its set-up stream, and no
+// graph captured there, takes the slots, every other application goes colour by colour.
+static bool one_launch(const Ctx& c, int cfg, int64_t ncols, size_t esize) {
+  if (cfg != 0 || !asm_fits(c, ncols, esize)) return false;
+  if ((c.terms & FE_KS_TERM_NL) && c.n_pairs > 0) return true;
+  if (c.stream != c.home_stream || c.stream == cudaStreamPerThread) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c.stream, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return cap == cudaStreamCaptureStatusNone;
+}
+
+// Cell part of an application: one launch for all cells and the sums of the shared
+// rows (one), or one launch per colour.
+template <typename T, typename TS>
+static cudaError_t launch_cells(const Ctx& c, LocalParams<T, TS>& lp, bool one, bool accum, int* launches,
+                                const std::function<cudaError_t()>& launch) {
+  cudaError_t err = cudaSuccess;
+  if (one) {
+    lp.cells = nullptr;
+    lp.n_cells = (int)c.E;
+    lp.dst = c.asm_dst;
+    lp.W = static_cast<TS*>(c.asm_W);
+    lp.accum = accum;
+    std::lock_guard<std::mutex> lk(c.asm_mu);   // another thread's pair of launches does not come between
+    err = launch();
+    if (err == cudaSuccess) err = launch_assemble<TS>(c, lp.Y, lp.ncols, accum, c.stream);
+    *launches += c.n_shared > 0 ? 2 : 1;
+    return err;
+  }
+  for (size_t col = 0; col + 1 < c.colour_ptr.size() && err == cudaSuccess; ++col) {
+    lp.cells = c.colour_cells + c.colour_ptr[col];
+    lp.n_cells = c.colour_ptr[col + 1] - c.colour_ptr[col];
+    if (lp.n_cells == 0) continue;
+    err = launch();
+    ++*launches;
+  }
+  return err;
+}
+
 template <typename T>
 fe_ks_status apply_core(Ctx& c, const T* X, T* Y, int64_t ncols, bool scaled, T alpha, bool zero_fill, int tc) {
   NvtxRange range(tc == 3   ? "fe_ks_apply bf16x2"
@@ -685,9 +814,11 @@ fe_ks_status apply_core(Ctx& c, const T* X, T* Y, int64_t ncols, bool scaled, T 
     c.ev_pool.pop_back();
     cudaEventRecord(ev[i], s);
   };
+  const bool one = !tc && one_launch(c, sizeof(T) == 8 ? c.cfg64 : c.cfg32, ncols, sizeof(T));
   mark(0);
-  if (zero_fill && cudaMemsetAsync(Y, 0, bytes, s) != cudaSuccess)
+  if (zero_fill && !one && cudaMemsetAsync(Y, 0, bytes, s) != cudaSuccess)
     return fail(FE_KS_ERR_CUDA, "cudaMemsetAsync failed");
+  if (one) nlaunch[0] = 0;
   mark(1);
   if (tc && c.nq != c.np)
     return fail(FE_KS_ERR_UNSUPPORTED, "the tensor-core precisions need n_q = n_p (square 1D operators)");
@@ -731,19 +862,18 @@ fe_ks_status apply_core(Ctx& c, const T* X, T* Y, int64_t ncols, bool scaled, T 
   lp.n_proj = c.n_proj;
   lp.alpha = alpha;
   lp.tab = od.tab;
-  for (size_t col = 0; col + 1 < c.colour_ptr.size(); ++col) {
-    lp.cells = c.colour_cells + c.colour_ptr[col];
-    lp.n_cells = c.colour_ptr[col + 1] - c.colour_ptr[col];
-    cudaError_t err;
-    if constexpr (std::is_same<T, float>::value)
-      err = !tc ? launch_local<T, T>(c, lp, s)   // tc: n_q = n_p, checked above
-            : use_tc5(c, tc) ? launch_tc5(c, lp, s, tc == 2, tc5_stagger(c.cfg_tc[tc - 1]))
-                             : launch_tc(c, lp, s, tc);
-    else
-      err = launch_local<T, T>(c, lp, s);
-    if (err != cudaSuccess) return fail(FE_KS_ERR_CUDA, std::string("local kernel: ") + cudaGetErrorString(err));
-    if (lp.n_cells > 0) nlaunch[2]++;
+  if constexpr (std::is_same<T, float>::value) {
+    lp.cell_coef = c.cell_coef;
+    for (int q = 0; q < c.nq; ++q) lp.w[q] = c.gauss_w[q];
   }
+  const cudaError_t err = launch_cells<T, T>(c, lp, one, !zero_fill, &nlaunch[2], [&]() -> cudaError_t {
+    if constexpr (std::is_same<T, float>::value) {
+      if (tc)   // n_q = n_p, checked above
+        return use_tc5(c, tc) ? launch_tc5(c, lp, s, tc == 2, tc5_stagger(c.cfg_tc[tc - 1])) : launch_tc(c, lp, s, tc);
+    }
+    return launch_local<T, T>(c, lp, s);
+  });
+  if (err != cudaSuccess) return fail(FE_KS_ERR_CUDA, std::string("local kernel: ") + cudaGetErrorString(err));
   mark(3);
   if (c.profiling) {
     c.ev_rec.push_back(ev);
@@ -776,8 +906,11 @@ fe_ks_status apply_core_emu(Ctx& c, const double* X, double* Y, int64_t ncols, b
     c.ev_pool.pop_back();
     cudaEventRecord(ev[i], s);
   };
+  const bool one = false;
   mark(0);
-  if (zero_fill && cudaMemsetAsync(Y, 0, bytes, s) != cudaSuccess) return fail(FE_KS_ERR_CUDA, "cudaMemsetAsync failed");
+  if (zero_fill && !one && cudaMemsetAsync(Y, 0, bytes, s) != cudaSuccess)
+    return fail(FE_KS_ERR_CUDA, "cudaMemsetAsync failed");
+  if (one) nlaunch[0] = 0;
   mark(1);
   const bool nl = (c.terms & FE_KS_TERM_NL) && c.n_pairs > 0;
   if (nl) {
@@ -819,13 +952,9 @@ fe_ks_status apply_core_emu(Ctx& c, const double* X, double* Y, int64_t ncols, b
   lp.n_proj = c.n_proj;
   lp.alpha = ff_from_double_host(alpha);
   lp.tab = c.emu.tab;
-  for (size_t col = 0; col + 1 < c.colour_ptr.size(); ++col) {
-    lp.cells = c.colour_cells + c.colour_ptr[col];
-    lp.n_cells = c.colour_ptr[col + 1] - c.colour_ptr[col];
-    cudaError_t err = launch_local<ff2, double>(c, lp, s);
-    if (err != cudaSuccess) return fail(FE_KS_ERR_CUDA, std::string("local kernel: ") + cudaGetErrorString(err));
-    if (lp.n_cells > 0) nlaunch[2]++;
-  }
+  const cudaError_t err = launch_cells<ff2, double>(c, lp, one, !zero_fill, &nlaunch[2],
+                                                    [&] { return launch_local<ff2, double>(c, lp, s); });
+  if (err != cudaSuccess) return fail(FE_KS_ERR_CUDA, std::string("local kernel: ") + cudaGetErrorString(err));
   mark(3);
   if (c.profiling) {
     c.ev_rec.push_back(ev);

@@ -5,6 +5,7 @@
 
 #include <array>
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -78,6 +79,15 @@ struct LocalParams {
   const TS* Q;             // [n_atoms][n_proj][ld], already scaled by Delta
   int n_proj;
   T alpha;                 // Y += alpha * (H X) (1 for a plain application)
+  // default kernel (fe_ks_line.cuh): one launch for all cells (cells = nullptr,
+  // dst: rows met by one cell are stored to Y, shared rows to their slots of W,
+  // summed by launch_assemble); axis-aligned cells (cell_coef: [E][8] scalars of
+  // the kinetic (0..2) and Bloch (4..6) coefficients, w: 1D Gauss weights)
+  const int* dst;
+  TS* W;
+  int accum;               // one launch: Y += instead of Y =
+  const T* cell_coef;
+  T w[kMaxN];
   EOTables<T> tab;
 };
 
@@ -101,6 +111,7 @@ struct ProjParams {
 };
 
 struct Ctx {
+  int sms = 0;                          // multiprocessors of the device
   int p = 0, nq = 0, np = 0, np3 = 0, nq3 = 0;
   int cplx = 0, terms = 0, gga = 0, ncoef = 0;
   int cfg64 = 0, cfg32 = 0, cfgE = 0;   // tile configuration of the fused kernel per precision
@@ -145,6 +156,20 @@ struct Ctx {
   uint4* tc5_cst16 = nullptr;      // the same in FP16
   int* dev_status = nullptr;       // device word: 1 after a bounded wait in a cell kernel expired
   int inject_fault = 0;            // host-side fault injection into the tcgen05 cell kernel (tests)
+  // axis-aligned cells (every cell a box): per-cell scalars of the FP32 default kernel, 1D Gauss weights
+  float* cell_coef = nullptr;
+  float gauss_w[kMaxN] = {};
+  // one-launch assembly: destination of every cell node (row of Y when one cell
+  // meets the DoF, else ~slot of W), the shared DoFs with their slot ranges, and
+  // the slots' values
+  int* asm_dst = nullptr;
+  int* asm_dof = nullptr;
+  int* asm_ptr = nullptr;    // [n_shared + 1]
+  int64_t n_shared = 0, n_wslots = 0;
+  void* asm_W = nullptr;
+  size_t asm_bytes = 0;
+  cudaStream_t home_stream = nullptr;   // of setup: the stream whose applications own the slots
+  mutable std::mutex asm_mu;
   std::vector<void*> allocations;
   // host-buffer pipeline (fe_ks_apply_host): copy-in and copy-out streams and,
   // per workspace slot, events for "X copied in", "applied", "Y copied out"
@@ -209,6 +234,18 @@ constexpr int kLocalConfigs = 10;
 // upper triangle of a symmetric product).
 constexpr int kGramChunkRows = 8192;
 cudaError_t launch_gram_reduce(const double* part, double* C, int nchunks, int n1, int n2, int upper, cudaStream_t s);
+
+// Column tiles per unit of work (a cell's tiles split evenly) for kernels whose blocks walk the tiles
+// of a cell: the fewest tile times over the units' rounds on `slots` resident blocks, a unit's start
+// (its cell's tables, an empty pipeline) costing `start` tiles.
+int tiles_per_unit(int64_t cells, int ntiles, int64_t slots, double start, int multiple = 1);
+// Y[dof] (+)= the DoF's slots of W, added in slot order (T = storage type)
+template <typename T>
+cudaError_t launch_assemble(const Ctx& c, T* Y, int64_t ncols, int accum, cudaStream_t s);
+// whether one application of ncols columns of the given storage size fits the slots
+inline bool asm_fits(const Ctx& c, int64_t ncols, size_t esize) {
+  return c.asm_dst && (size_t)c.n_wslots * (size_t)ncols * esize <= c.asm_bytes;
+}
 
 // kernel launchers (fe_ks_local_pN.cu)
 template <typename T, typename TS>

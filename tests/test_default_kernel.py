@@ -1,0 +1,131 @@
+"""The default cell kernels (tile configuration 0: line kernels, one-launch assembly) against the oracle
+at the sizes where their tiles, column forms and assembly can go wrong.
+
+* Column counts: one column (a tile holds several cells), counts below, at and above a
+  tile of every degree, odd counts (no 8-byte rows), counts that leave a partial tile;
+  real and complex, with the staged (16-byte rows) and the unstaged gather.
+* Axis-aligned cells (per-cell scalars) and jittered ones (per-point coefficients).
+* n_q = n_p + 2, the scaled form, and projectors on cells of several column tiles.
+* The one-launch assembly gives the same bits twice, and the bits of the
+  colour-by-colour scatter (which a stream other than the set-up one takes for an operator
+  without projectors).
+
+Tolerances as in test_parity_apply: 1e-12 for FP64 and pairs of floats, 1e-5 for FP32, per
+column and per entry.
+"""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from paper_2512_08571_gb300 import fe_ks as fk
+from synth.host_problem import HostProblem
+from oracle.operator import Problem
+from synth import Workload, trial_vectors
+from gpu_util import gpu_apply, parity_err, round_input
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = {fk.FE_KS_F64: 1e-12, fk.FE_KS_F32: 1e-5, fk.FE_KS_F64E: 1e-12}
+PREC = [fk.FE_KS_F64, fk.FE_KS_F32, fk.FE_KS_F64E]
+COLUMNS = (1, 2, 3, 7, 8, 12, 19, 32, 33)   # tiles hold 4..32 FP32 columns, 2..16 FP64 ones
+
+
+def _wl(p, cplx, jitter, nqx=0, n=2, n_atoms=2, n_v=max(COLUMNS)):
+    return Workload(f"line{p}{cplx}{jitter}", L=4.0 * n / 2, n=n, p=p, nq=p + 1 + nqx, n_v=n_v, jitter=jitter, gga=True,
+                    kfrac=(0.2, 0.1, -0.3) if cplx else (0.0, 0.0, 0.0), complex=cplx, n_atoms=n_atoms, seed=7700 + p)
+
+
+@pytest.mark.parametrize("jitter", [0.0, 0.08])
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5, 6, 7, 8])
+def test_columns_and_degrees(p, cplx, jitter):
+    wl = _wl(p, cplx, jitter, n=3 if p < 3 else 2)
+    hp, X = HostProblem(wl), trial_vectors(wl)
+    P = Problem(wl)
+    Yref64, Yref32 = P.apply(X), P.apply(round_input(X, fk.FE_KS_F32))
+    for precision in PREC:
+        for nv in COLUMNS:
+            Y = gpu_apply(hp, np.ascontiguousarray(round_input(X, precision)[:, :nv]), precision)
+            ref = (Yref32 if precision == fk.FE_KS_F32 else Yref64)[:, :nv]
+            assert parity_err(Y, ref) <= TOL[precision], (precision, nv)
+
+
+@pytest.mark.parametrize("jitter", [0.0, 0.08])
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5, 6, 7, 8])
+def test_full_tiles(p, cplx, jitter):
+    """As many columns as give every multiprocessor one full tile (the kernels take tiles of two
+    elements below that), less a few so that the last tile of a cell is partial and, for real
+    FP32, rows are not 8-byte aligned; the FP32 case runs the wide form (a block per cell)."""
+    n = 3 if p < 3 else 2
+    vg = 16 if p < 4 else 8 if p < 6 else 4
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    elems = sms * vg // n ** 3 - 1
+    cols = {fk.FE_KS_F64: elems, fk.FE_KS_F64E: elems, fk.FE_KS_F32: 2 * elems - (0 if cplx else 1)}
+    nvs = {k: v // 2 if cplx else v for k, v in cols.items()}
+    wl = _wl(p, cplx, jitter, n=n, n_v=max(nvs.values()))
+    hp, X = HostProblem(wl), trial_vectors(wl)
+    P = Problem(wl)
+    ref = P.apply(X)
+    for precision in PREC:
+        Xin = np.ascontiguousarray(round_input(X, precision)[:, :nvs[precision]])
+        Y = gpu_apply(hp, Xin, precision)
+        want = P.apply(Xin) if precision == fk.FE_KS_F32 else ref[:, :nvs[precision]]
+        assert parity_err(Y, want) <= TOL[precision], precision
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("p", [4, 6, 7, 8])
+def test_more_points_than_nodes_and_scaled(p, cplx):
+    wl = _wl(p, cplx, 0.05, nqx=2, n_v=9)
+    hp, X = HostProblem(wl), trial_vectors(wl)
+    P = Problem(wl)
+    s = 1.0 / np.sqrt(P.lumped_mass())
+    for precision in PREC:
+        Xin = round_input(X, precision)
+        ref = s[:, None] * P.apply(s[:, None] * Xin)
+        for nv in (1, 8, 9):
+            Y = gpu_apply(hp, np.ascontiguousarray(Xin[:, :nv]), precision, scaled=True)
+            assert parity_err(Y, ref[:, :nv]) <= TOL[precision], (precision, nv)
+
+
+@pytest.mark.parametrize("precision", PREC[:2])
+def test_same_bits_twice(precision):
+    wl = dataclasses.replace(_wl(6, False, 0.05, n=3), n_v=21)
+    hp, X = HostProblem(wl), round_input(trial_vectors(wl), precision)
+    a, b = gpu_apply(hp, X, precision, repeat=2)
+    assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("precision", PREC[:2])
+def test_one_launch_gives_the_bits_of_the_colour_launches(precision):
+    """Operator without projectors: the set-up stream takes the one-launch assembly, another
+    stream and a captured graph go colour by colour; all the same bits."""
+    wl = _wl(5, False, 0.05, n=3, n_atoms=0, n_v=13)
+    hp = HostProblem(wl)
+    dt = torch.float32 if precision == fk.FE_KS_F32 else torch.float64
+    X = torch.from_numpy(trial_vectors(wl)).cuda().to(dt)
+    ys = [torch.full_like(X, float("nan")) for _ in range(3)]
+    side = torch.cuda.Stream()
+    home = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    ctx = fk.fe_ks_setup(hp.struct, fk.TERM_ALL, wl.n_v, home.cuda_stream)
+    try:
+        fk.fe_ks_apply(ctx, X, ys[0], wl.n_v, precision)
+        fk.fe_ks_set_stream(ctx, side.cuda_stream)
+        fk.fe_ks_apply(ctx, X, ys[1], wl.n_v, precision)
+        torch.cuda.synchronize()
+        fk.fe_ks_set_stream(ctx, home.cuda_stream)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.stream(home):
+            graph.capture_begin()
+            fk.fe_ks_apply(ctx, X, ys[2], wl.n_v, precision)
+            graph.capture_end()
+        graph.replay()
+        torch.cuda.synchronize()
+    finally:
+        fk.fe_ks_destroy(ctx)
+    assert not torch.isnan(ys[0]).any()
+    assert torch.equal(ys[0], ys[1]) and torch.equal(ys[0], ys[2])
