@@ -943,12 +943,10 @@ cudaError_t launch_n(Params p, cudaStream_t s) {
   cudaError_t err = cudaFuncSetAttribute(fe_tc5_kernel<N, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::BYTES);
   if (err != cudaSuccess) return err;
   const int ntiles = (p.ncols + G::VT - 1) / G::VT;
-  // split a cell's column tiles into units so that every SM gets about 16 or more;
-  // a unit's tiles alternate between the CTA's two pipelines, so keep the count even
-  int upc = 1;
-  while (2 * upc < ntiles && (int64_t)p.n_cells * upc < 16LL * sms) upc *= 2;
-  p.tiles_per_unit = (ntiles + upc - 1) / upc;
-  p.tiles_per_unit += p.tiles_per_unit & 1;
+  // units of column tiles of one cell: even (the tiles alternate between the CTA's two pipelines),
+  // a unit's start (coefficients, first gather and plane product, drained pipelines) costing
+  // about three tiles
+  p.tiles_per_unit = tiles_per_unit(p.n_cells, ntiles, sms, 3.0, 2);
   p.units_per_cell = (ntiles + p.tiles_per_unit - 1) / p.tiles_per_unit;
   const int64_t units = (int64_t)p.n_cells * p.units_per_cell;
   const int grid = (int)std::min<int64_t>(units, sms);
