@@ -6,7 +6,10 @@
 //                    partials F^(a,e)^H X^(e) (eq. AXmatrixfreenonloc, first factor),
 //   phase 1        : per-atom sums of the partials in pair order, scaled by Delta
 //                    (systems with projectors only),
-//   phase o + c    : the cells of colour c of every system (o = 2 with
+//   phase 2        : systems with projectors whose slots (fe_ks_assemble.cu) hold the
+//                    columns: every cell, shared rows to their slots; phase 3: the
+//                    sums of the shared rows.  Nothing to zero-fill.
+//   phase o + c    : otherwise the cells of colour c of every system (o = 2 with
 //                    projectors, 1 without; Algorithm 2 on a tile of cells x
 //                    columns, expansion and scatter-add fused).
 // Persistent CTAs claim items in queue order with one atomic counter.  An
@@ -32,6 +35,7 @@
 // overlap.  Items still wait only on earlier items of their own system, which
 // sit in the same queue.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <numeric>
 #include <vector>
@@ -145,6 +149,14 @@ static constexpr int kStateWords = 3 + kMaxSys * kMaxPhase;
 
 static bool batch_split(const fe_ks_batch* b) { return b->split_nt[0] > 0 && b->split_nt[1] > 0; }
 
+// One cell phase for all colours, through the context's slots: systems with projectors only
+// (their contexts have per-application scratch, Q, in any case; one without projectors may be
+// applied elsewhere while the batch runs).  Eight colour phases of FP64 tiles, each a dependent
+// step of at least one tile's time, were most of a batch of small systems.
+static bool batch_slots(const Ctx& c, int64_t ncols, int prec) {
+  return (c.terms & FE_KS_TERM_NL) && c.n_pairs > 0 && asm_fits(c, ncols, prec == FE_KS_F64 ? 8 : 4);
+}
+
 static fe_ks_status batch_build(fe_ks_batch* b) {
   std::vector<int4> items;
   std::vector<int> need(kMaxSys * kMaxPhase, 0);
@@ -153,7 +165,7 @@ static fe_ks_status batch_build(fe_ks_batch* b) {
   int max_ph = 0;
   for (int s = 0; s < ns; ++s)
     if (b->direct.empty() || !b->direct[s])
-      max_ph = std::max<int>(max_ph, (int)b->ctxs[s]->c.colour_ptr.size() - 1 + 2);
+      max_ph = std::max<int>(max_ph, std::max<int>(4, (int)b->ctxs[s]->c.colour_ptr.size() - 1 + 2));
   if (max_ph >= kMaxPhase) return fail(FE_KS_ERR_UNSUPPORTED, "too many colours for the batched launch");
   std::vector<std::vector<int4>> per_phase(max_ph + 1);
   std::vector<std::vector<int4>> per_phase_cls[2] = {std::vector<std::vector<int4>>(max_ph + 1),
@@ -172,13 +184,14 @@ static fe_ks_status batch_build(fe_ks_batch* b) {
     const size_t cb = b->prec[s] == FE_KS_F64 ? cell_bytes<double>(c.p, b->cfg[s]) : cell_bytes<float>(c.p, b->cfg[s]);
     if (cb == 0 || cb > 227 * 1024) return fail(FE_KS_ERR_UNSUPPORTED, "tile configuration does not fit");
     sm = std::max(sm, cb);
-    // phase 0: zero-fill slices and projections
+    const bool nl = (c.terms & FE_KS_TERM_NL) && c.n_pairs > 0;
+    const bool slots = batch_slots(c, ncols, b->prec[s]);
+    // phase 0: zero-fill slices (colour phases only) and projections
     const int rows = std::max(1, 65536 / ncols);
-    for (int64_t r = 0; r < c.m; r += rows) {
+    for (int64_t r = 0; !slots && r < c.m; r += rows) {
       pp[0].push_back(make_int4(s | (kItemZero << 8), (int)r, 0, (int)std::min<int64_t>(rows, c.m - r)));
       need[s * kMaxPhase + 0]++;
     }
-    const bool nl = (c.terms & FE_KS_TERM_NL) && c.n_pairs > 0;
     if (nl) {
       const int cw = batch_proj_cw(ncols, nt);
       sm = std::max(sm, b->prec[s] == FE_KS_F64 ? batch_proj_bytes<double>(c.n_proj, c.np3, cw, nt)
@@ -194,6 +207,19 @@ static fe_ks_status batch_build(fe_ks_batch* b) {
           need[s * kMaxPhase + 1]++;
         }
     }
+    if (slots) {   // phase 2: every cell; phase 3: the sums of the shared rows
+      for (int c0 = 0; c0 < (int)c.E; c0 += b->cells_per_item)
+        for (int t = 0; t < ncols; t += vt) {
+          pp[2].push_back(make_int4(s | (kItemLocal << 8) | (2 << 16), c0, t, std::min<int>(b->cells_per_item, (int)c.E - c0)));
+          need[s * kMaxPhase + 2]++;
+        }
+      const int arows = std::max(1, 16384 / ncols);
+      for (int64_t r = 0; r < c.n_shared; r += arows) {
+        pp[3].push_back(make_int4(s | (kItemAsm << 8) | (3 << 16), (int)r, 0, (int)std::min<int64_t>(arows, c.n_shared - r)));
+        need[s * kMaxPhase + 3]++;
+      }
+      continue;
+    }
     const int ph0 = nl ? 2 : 1;   // no empty phase: a colour waits on the phase just before it
     for (int col = 0; col + 1 < (int)c.colour_ptr.size(); ++col) {
       const int ph = col + ph0;
@@ -206,6 +232,19 @@ static fe_ks_status batch_build(fe_ks_batch* b) {
       }
     }
   }
+  // the longest cell items of a phase first (FP64 ones cost about 40 FP32 ones), so that a phase ends evenly
+  auto cost = [&](const int4& w) -> double {
+    if (((w.x >> 8) & 0xff) != kItemLocal) return 0.0;
+    const Ctx& c = b->ctxs[w.x & 0xff]->c;
+    return (b->prec[w.x & 0xff] == FE_KS_F64 ? 40.0 : 1.0) * std::pow((double)c.nq, 4) * vt_of(c.p, b->cfg[w.x & 0xff]) * w.w;
+  };
+  auto longest_first = [&](std::vector<std::vector<int4>>& pp) {
+    for (auto& v : pp)
+      std::stable_sort(v.begin(), v.end(), [&](const int4& a, const int4& c) { return cost(a) > cost(c); });
+  };
+  longest_first(per_phase);
+  longest_first(per_phase_cls[0]);
+  longest_first(per_phase_cls[1]);
   if (b->inject_missing) need[0]++;   // host-side fault injection: one item that is never published
   cudaMemcpy(b->d_need, need.data(), need.size() * sizeof(int), cudaMemcpyHostToDevice);
   auto upload_items = [&](const std::vector<int4>& v, int4** dst) -> bool {
@@ -276,6 +315,11 @@ static fe_ks_status batch_build(fe_ks_batch* b) {
     d.part = f64 ? (void*)c.f64.part : (void*)c.f32.part;
     d.n_proj = c.n_proj;
     d.np3 = c.np3;
+    const bool slots = batch_slots(c, d.ncols, b->prec[s]);
+    d.dst = slots ? c.asm_dst : nullptr;
+    d.W = c.asm_W;
+    d.asm_dof = c.asm_dof;
+    d.asm_ptr = c.asm_ptr;
     build_eo_tables<double>(c.p, c.nq, &P.t64[c.p]);
     build_eo_tables<float>(c.p, c.nq, &P.t32[c.p]);
   }

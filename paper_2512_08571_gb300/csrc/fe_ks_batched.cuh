@@ -16,7 +16,7 @@ constexpr int kBatchThreads[4] = {384, 512, 672, 256};
 // Precision classes of a kernel object: every routine, or the FP64 / FP32 ones
 // only (a split batch runs one persistent launch per class, concurrently).
 enum : int { kClassAll = 0, kClassF64 = 1, kClassF32 = 2 };
-enum : int { kItemZero = 0, kItemPair = 1, kItemLocal = 2, kItemSum = 3 };
+enum : int { kItemZero = 0, kItemPair = 1, kItemLocal = 2, kItemSum = 3, kItemAsm = 4 };
 
 
 struct BatchSys {
@@ -43,6 +43,11 @@ struct BatchSys {
   void* part;      // projection partials [pair][n_proj][ncols]
   int n_proj;
   int np3;
+  // one cell phase for all colours (systems with projectors whose slots hold ncols columns), else dst = nullptr
+  const int* dst;
+  void* W;
+  const int* asm_dof;
+  const int* asm_ptr;
 };
 
 struct BatchParams {
@@ -62,6 +67,7 @@ struct BatchParams {
 // Operand view of one system for the cell routine (field names of LocalParams).
 template <typename T>
 struct SysArgs {
+  static constexpr bool kSlots = true;
   const T* X;
   T* Y;
   int64_t ld;
@@ -78,6 +84,8 @@ struct SysArgs {
   const T* Q;
   int n_proj;
   T alpha;
+  const int* dst;
+  T* W;
 };
 
 template <typename T>
@@ -99,6 +107,8 @@ __device__ __forceinline__ SysArgs<T> sys_args(const BatchSys& s) {
   a.Q = static_cast<const T*>(s.Q);
   a.n_proj = s.n_proj;
   a.alpha = T(1);
+  a.dst = s.dst;
+  a.W = static_cast<T*>(s.W);
   return a;
 }
 
@@ -107,6 +117,20 @@ __device__ void zero_item(const BatchSys& s, int row0, int rows) {
   T* Y = static_cast<T*>(s.Y) + (int64_t)row0 * s.ncols;
   const int64_t n = (int64_t)rows * s.ncols;
   for (int64_t i = threadIdx.x; i < n; i += blockDim.x) Y[i] = T(0);
+}
+
+// Rows [r0, r0 + rows) of the shared DoFs: Y[dof] = the DoF's slots, added in slot order
+template <typename T>
+__device__ void asm_item(const BatchSys& s, int r0, int rows) {
+  T* Y = static_cast<T*>(s.Y);
+  const T* W = static_cast<const T*>(s.W);
+  for (int i = threadIdx.x; i < rows * s.ncols; i += blockDim.x) {
+    const int r = r0 + i / s.ncols, col = i % s.ncols;
+    const int b = s.asm_ptr[r], e = s.asm_ptr[r + 1];
+    T v = W[(int64_t)b * s.ncols + col];
+    for (int k = b + 1; k < e; ++k) v += W[(int64_t)k * s.ncols + col];
+    Y[(int64_t)s.asm_dof[r] * s.ncols + col] = v;
+  }
 }
 
 // Columns per projection item: the smallest of 32, 64, 128 that covers the
@@ -265,6 +289,8 @@ __global__ void __launch_bounds__(NT, MINB) fe_batched_kernel(const __grid_const
         if constexpr (CLS != kClassF32) {
           if (kind == kItemZero)
             zero_item<double>(s, w.y, w.w);
+          else if (kind == kItemAsm)
+            asm_item<double>(s, w.y, w.w);
           else if (kind == kItemPair)
             pair_item<double, NT>(s, w.y, w.z, w.w, smem);
           else if (kind == kItemSum)
@@ -276,6 +302,8 @@ __global__ void __launch_bounds__(NT, MINB) fe_batched_kernel(const __grid_const
         if constexpr (CLS != kClassF64) {
           if (kind == kItemZero)
             zero_item<float>(s, w.y, w.w);
+          else if (kind == kItemAsm)
+            asm_item<float>(s, w.y, w.w);
           else if (kind == kItemPair)
             pair_item<float, NT>(s, w.y, w.z, w.w, smem);
           else if (kind == kItemSum)

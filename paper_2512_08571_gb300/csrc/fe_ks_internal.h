@@ -60,6 +60,7 @@ struct OpData {
 // (they differ only for the pair-of-floats FP64 variant).
 template <typename T, typename TS = T>
 struct LocalParams {
+  static constexpr bool kSlots = false;   // the routines of fe_ks_local.cuh scatter colour by colour
   const TS* X;
   TS* Y;
   int64_t ld;              // row pitch of X and Y in scalars (= ncols)

@@ -436,6 +436,13 @@ __device__ __forceinline__ void tile_body(const Prm& p, const EOTables<T>& tb, i
       const int d = sd[i + NP * (j + NP * k)];
       T val = y[i] * p.alpha;
       if (p.dscale) val *= p.dscale[d];
+      if constexpr (Prm::kSlots) {
+        if (p.dst) {   // all cells at once: rows of one cell straight to Y, shared rows to their slots
+          const int q = p.dst[(int64_t)e * NP3 + i + NP * (j + NP * k)];
+          *(q >= 0 ? p.Y + (int64_t)q * p.ld + col : p.W + (int64_t)(~q) * p.ld + col) = val;
+          continue;
+        }
+      }
       auto* yp = p.Y + (int64_t)d * p.ld + col;
       if constexpr (ATOMIC)
         atomicAdd(yp, val);   // fire-and-forget reduction; the colouring keeps it race-free anyway
