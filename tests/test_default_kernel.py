@@ -6,7 +6,7 @@ at the sizes where their tiles, column forms and assembly can go wrong.
   real and complex, with the staged (16-byte rows) and the unstaged gather.
 * Axis-aligned cells (per-cell scalars) and jittered ones (per-point coefficients).
 * n_q = n_p + 2, the scaled form, and projectors on cells of several column tiles.
-* The one-launch assembly gives the same bits twice, and the bits of the
+* The one-launch assembly gives the same bits twice, in every precision, and the bits of the
   colour-by-colour scatter (which a stream other than the set-up one takes for an operator
   without projectors).
 
@@ -91,7 +91,7 @@ def test_more_points_than_nodes_and_scaled(p, cplx):
             assert parity_err(Y, ref[:, :nv]) <= TOL[precision], (precision, nv)
 
 
-@pytest.mark.parametrize("precision", PREC[:2])
+@pytest.mark.parametrize("precision", PREC)
 def test_same_bits_twice(precision):
     wl = dataclasses.replace(_wl(6, False, 0.05, n=3), n_v=21)
     hp, X = HostProblem(wl), round_input(trial_vectors(wl), precision)
@@ -99,7 +99,7 @@ def test_same_bits_twice(precision):
     assert np.array_equal(a, b)
 
 
-@pytest.mark.parametrize("precision", PREC[:2])
+@pytest.mark.parametrize("precision", PREC)
 def test_one_launch_gives_the_bits_of_the_colour_launches(precision):
     """Operator without projectors: the set-up stream takes the one-launch assembly, another
     stream and a captured graph go colour by colour; all the same bits."""
