@@ -187,7 +187,9 @@ bool line_small(int64_t slots, int sms) {
   return 8 * small <= 7 * full;
 }
 
-// Shared memory of the wide form after the three tiles: [X tile] [coefficients] [DoFs] [destinations]
+// Shared memory of the wide form after the three tiles: [coefficients] [DoFs] [destinations] [a pair's
+// projections Q of the tile's columns] [X tile].  A pair's F block takes tiles B and C, free in h and i.
+constexpr int kLineMaxProj = 16;   // projectors an atom can carry
 template <int NP, int NQ, bool CPLX, bool BOX>
 struct WideShape {
   using S = LineShape<NQ>;
@@ -195,7 +197,8 @@ struct WideShape {
   static constexpr int NCF = BOX ? 4 : CPLX ? kCoefCplx : kCoefReal;   // coefficient rows kept (BOX: V_L, V_G)
   static constexpr size_t cf = ((size_t)NCF * NQ3 * 4 + 15) / 16 * 16, idx = ((size_t)NP3 * 4 + 15) / 16 * 16;
   static constexpr size_t xs = (size_t)NP3 * S::VG * 8;
-  static constexpr size_t rest = S::tiles + cf + 2 * idx;
+  static constexpr size_t qs = (size_t)kLineMaxProj * S::VG * 8;
+  static constexpr size_t rest = S::tiles + cf + 2 * idx + qs;
   static constexpr bool STAGE_X = (rest + xs + 1024) * S::MINB <= 228 * 1024;
   static constexpr size_t bytes = rest + (STAGE_X ? xs : 0);
   static constexpr int MINB = (bytes + 1024) * S::MINB <= 228 * 1024 ? S::MINB : S::MINB - 1;
@@ -228,6 +231,12 @@ __global__ void __launch_bounds__(LineShape<NQ, FORM == kLineSmall>::NT, line_bl
   [[maybe_unused]] float* const cfs = reinterpret_cast<float*>(smem_raw + S::tiles);
   [[maybe_unused]] int* const sdof = reinterpret_cast<int*>(smem_raw + S::tiles + W::cf);
   [[maybe_unused]] int* const sdst = reinterpret_cast<int*>(smem_raw + S::tiles + W::cf + W::idx);
+  [[maybe_unused]] float* const qs = reinterpret_cast<float*>(smem_raw + S::tiles + W::cf + 2 * W::idx);
+  [[maybe_unused]] float* const Fs = reinterpret_cast<float*>(smem_raw + (size_t)S::BUF * 8);
+  constexpr int CW = CPLX ? 2 : 1;
+  // wide form: a pair's F block fits tiles B and C
+  [[maybe_unused]] const bool fits_f = (size_t)p.n_proj * NP3 * CW * sizeof(float) <= 2 * (size_t)S::BUF * 8;
+  [[maybe_unused]] int pbeg = 0, pend = 0, pair0 = 0, atom0 = 0;   // wide form: the cell's pairs, its first one
   [[maybe_unused]] V* const XS = reinterpret_cast<V*>(smem_raw + W::rest);
   const bool node_line = ln < NP2, gauss_line = ln < NQ2, mixed_line = ln < NP * NQ;
   const unsigned gmask = CPLX ? __ballot_sync(0xffffffffu, gauss_line) : 0u;
@@ -263,9 +272,24 @@ __global__ void __launch_bounds__(LineShape<NQ, FORM == kLineSmall>::NT, line_bl
     }
   };
 
-  // one tile: cell e, first column col of this lane; act: the lane stores.  next: called once phase a
-  // has read the tile's rows of X
-  auto tile = [&](int e, int col, bool act, auto next) {
+  // a pair's F block -> B and C, and its projections of column elements [c0, c0 + VG) -> qs
+  [[maybe_unused]] auto stage_f = [&](int pr, int atom, int c0) {
+    if constexpr (WIDE) {
+      const float* F = p.F + (int64_t)pr * p.n_proj * NP3 * CW;
+      for (int i = threadIdx.x; i < p.n_proj * NP3 * CW; i += NT) cp_async_4(Fs + i, F + i);
+      const float* Q = p.Q + (int64_t)atom * p.n_proj * p.ld;
+      for (int i = threadIdx.x; i < p.n_proj * 2 * VG; i += NT) {
+        const int col = 2 * c0 + i % (2 * VG);
+        const bool in = col < p.ncols;
+        cp_async_4z(qs + i, in ? Q + (int64_t)(i / (2 * VG)) * p.ld + col : Q, in ? 4 : 0);
+      }
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+  };
+
+  // one tile: cell e, first column col of this lane; act: the lane stores; c0: the tile's first
+  // column element (wide form).  next: called once phase a has read the tile's rows of X
+  auto tile = [&](int e, int col, bool act, [[maybe_unused]] int c0, auto next) {
     const bool two = CPE == 1 || col + 1 < p.ncols;
     // a
     if (node_line) {
@@ -407,6 +431,8 @@ __global__ void __launch_bounds__(LineShape<NQ, FORM == kLineSmall>::NT, line_bl
       for (int i = 0; i < NP; ++i) A[ox + i * SX] = y[i];
     }
     __syncthreads();
+    const bool staged_f = WIDE && pend > pbeg && fits_f;
+    if (staged_f) stage_f(pair0, atom0, c0);   // arrives behind h
     // h
     if (mixed_line) {
       V x[NQ], y[NP];
@@ -416,14 +442,48 @@ __global__ void __launch_bounds__(LineShape<NQ, FORM == kLineSmall>::NT, line_bl
 #pragma unroll
       for (int j = 0; j < NP; ++j) A[om + j * SY] = y[j];
     }
+    if (staged_f) asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
     // i
-    if (node_line && act) {
-      V x[NQ], y[NP];
+    V y[NP];
+    if (node_line) {
+      V x[NQ];
 #pragma unroll
       for (int q = 0; q < NQ; ++q) x[q] = A[on + q * SZ];
       eo_apply<NQ, NP, 1>(x, y, tab.Nt);
-      if (p.cell_pair_ptr) {
+    }
+    if constexpr (WIDE) {
+      if (staged_f)
+        for (int pi = pbeg;;) {
+          if (node_line) {
+#pragma unroll 3
+            for (int b = 0; b < p.n_proj; ++b) {
+              V q;
+              q.v = *reinterpret_cast<const unsigned long long*>(qs + (b * VG + v) * 2);
+              if constexpr (!CPLX) {
+#pragma unroll
+                for (int k = 0; k < NP; ++k) y[k] = fma(Fs[b * NP3 + ln + k * NP2], q, y[k]);
+              } else {
+                const float2 s = f2v_split(q);
+                const V iq = f2v_make(-s.y, s.x);
+#pragma unroll
+                for (int k = 0; k < NP; ++k) {
+                  const float2 f = *reinterpret_cast<const float2*>(Fs + (b * NP3 + ln + k * NP2) * 2);
+                  y[k] = fma(f.x, q, fma(f.y, iq, y[k]));
+                }
+              }
+            }
+          }
+          if (++pi >= pend) break;
+          __syncthreads();   // the next pair of the cell takes the same place
+          const int pr = p.cell_pairs[pi];
+          stage_f(pr, p.pair_atom[pr], c0);
+          asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+          __syncthreads();
+        }
+    }
+    if (node_line && act) {
+      if (p.cell_pair_ptr && !staged_f) {
         const int pb = p.cell_pair_ptr[e], pe = p.cell_pair_ptr[e + 1];
         for (int pi = pb; pi < pe; ++pi) {
           const int pr = p.cell_pairs[pi];
@@ -507,6 +567,10 @@ __global__ void __launch_bounds__(LineShape<NQ, FORM == kLineSmall>::NT, line_bl
         const T* g = p.coef + ((int64_t)e * p.ncoef + (BOX ? 6 : 0)) * NQ3;
         for (int i = threadIdx.x; i < W::NCF * NQ3; i += NT) cp_async_4(cfs + i, g + i);
         asm volatile("cp.async.commit_group;\n" ::: "memory");
+        if (p.cell_pair_ptr) {
+          pbeg = p.cell_pair_ptr[e], pend = p.cell_pair_ptr[e + 1];
+          if (pend > pbeg) pair0 = p.cell_pairs[pbeg], atom0 = p.pair_atom[pair0];
+        }
         staged = ci;
         __syncthreads();
       }
@@ -517,7 +581,7 @@ __global__ void __launch_bounds__(LineShape<NQ, FORM == kLineSmall>::NT, line_bl
           __syncthreads();
         }
         const bool act = t * VG + v < ncg;
-        tile(e, act ? (t * VG + v) * CPE : 0, act, [&] {
+        tile(e, act ? (t * VG + v) * CPE : 0, act, t * VG, [&] {
           if constexpr (W::STAGE_X)
             if (t + 1 < te) stage_x((t + 1) * VG);
         });
@@ -531,7 +595,7 @@ __global__ void __launch_bounds__(LineShape<NQ, FORM == kLineSmall>::NT, line_bl
       const bool act = slot < nslots;
       const int ci = act ? (int)(slot / ncg) : p.n_cells - 1;
       const int ce = act ? (int)(slot - (int64_t)ci * ncg) : (CPLX && CPE == 1) ? (int)(slot & 1) : 0;
-      tile(p.cells ? p.cells[ci] : ci, ce * CPE, act, [] {});
+      tile(p.cells ? p.cells[ci] : ci, ce * CPE, act, 0, [] {});
     }
   }
 }
