@@ -269,18 +269,23 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_partial(const double* __res
   }
 }
 
-// out = sum of part (sqrt if root); one warp, fixed order
-__global__ void k_dot_final(const double* __restrict__ part, double* __restrict__ out, int root) {
+// out = sum of part (sqrt if root, and its reciprocal to inv); one warp, fixed order
+__global__ void k_dot_final(const double* __restrict__ part, double* __restrict__ out, double* __restrict__ inv,
+                            int root) {
   double s = 0.0;
   for (int i = threadIdx.x; i < kRedBlocks; i += 32) s += part[i];
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-  if (threadIdx.x == 0) *out = root ? sqrt(s) : s;
+  if (threadIdx.x == 0) {
+    const double r = root ? sqrt(s) : s;
+    *out = r;
+    if (inv) *inv = 1.0 / r;
+  }
 }
 
-// v = x / *nrm
-__global__ void k_scale_by_inv(double* __restrict__ v, const double* __restrict__ x, const double* __restrict__ nrm,
+// v = x *inv (an FP64 division per thread took 10 us for a vector of 7 MB, the copy 3)
+__global__ void k_scale_by_inv(double* __restrict__ v, const double* __restrict__ x, const double* __restrict__ inv,
                                int64_t n) {
-  const double r = 1.0 / *nrm;
+  const double r = *inv;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     v[i] = x[i] * r;
 }
@@ -296,10 +301,10 @@ __global__ void k_lanczos_orth(double* __restrict__ w, const double* __restrict_
   }
 }
 
-static void dot_device(const double* a, const double* b, int64_t n, double* part, double* out, bool root,
+static void dot_device(const double* a, const double* b, int64_t n, double* part, double* out, double* inv, bool root,
                        cudaStream_t s) {
   k_dot_partial<<<kRedBlocks, kRedThreads, 0, s>>>(a, b, n, part);
-  k_dot_final<<<1, 32, 0, s>>>(part, out, root ? 1 : 0);
+  k_dot_final<<<1, 32, 0, s>>>(part, out, inv, root ? 1 : 0);
 }
 
 // Largest eigenvalue of the symmetric tridiagonal matrix (diag a[0..k-1], off-diagonal b[0..k-2])
@@ -664,16 +669,17 @@ fe_ks_status fe_ks_lanczos_bound(fe_ks_ctx* ctx, const double* v0, int steps, in
   }
   const int ew = (int)std::min<int64_t>((n + 255) / 256, 152 * 16);
   // v = v0 / |v0|  (the norm goes to beta[steps] as scratch)
-  dot_device(v0, v0, n, part, dbe + steps, true, s);
-  k_scale_by_inv<<<ew, 256, 0, s>>>(v, v0, dbe + steps, n);
+  double* inv = dal + steps;   // the last reciprocal norm
+  dot_device(v0, v0, n, part, dbe + steps, inv, true, s);
+  k_scale_by_inv<<<ew, 256, 0, s>>>(v, v0, inv, n);
   for (int i = 0; i < steps; ++i) {
     st = fe_ks_apply_scaled(ctx, v, wv, 1, precision);
     if (st != FE_KS_OK) return st;
-    dot_device(v, wv, n, part, dal + i, false, s);
+    dot_device(v, wv, n, part, dal + i, nullptr, false, s);
     k_lanczos_orth<<<ew, 256, 0, s>>>(wv, v, vp, dal + i, i > 0 ? dbe + i - 1 : nullptr, n);
-    dot_device(wv, wv, n, part, dbe + i, true, s);
+    dot_device(wv, wv, n, part, dbe + i, inv, true, s);
     std::swap(v, vp);                                        // vp <- v (old)
-    k_scale_by_inv<<<ew, 256, 0, s>>>(v, wv, dbe + i, n);    // v <- w / beta
+    k_scale_by_inv<<<ew, 256, 0, s>>>(v, wv, inv, n);    // v <- w / beta
   }
   if ((st = last_cuda("Lanczos kernels")) != FE_KS_OK) return st;
   std::vector<double> a(steps), b(steps);
