@@ -360,7 +360,7 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
   // axis-aligned box cells: J diagonal and constant over the cell (to well below FP32
   // rounding), so the kinetic and Bloch coefficients are a scalar of the cell times
   // the point's weight
-  std::vector<float> cell_coef((size_t)E * 8, 0.f);
+  std::vector<float> cell_coef((size_t)E * 16, 0.f);
   std::atomic<int> boxes(1);
   parallel_for(E, [&](int64_t b, int64_t e_end) {
     for (int64_t e = b; e < e_end; ++e) {
@@ -408,9 +408,13 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
       if (!box) boxes.store(0, std::memory_order_relaxed);
       if (box) {
         const double det = J0[0] * J0[1] * J0[2];
+        auto put = [&](int k, double v) {
+          cell_coef[e * 16 + k] = (float)v;
+          cell_coef[e * 16 + 8 + k] = (float)(v - (double)(float)v);
+        };
         for (int s = 0; s < 3; ++s) {
-          if (terms_mask & FE_KS_TERM_T) cell_coef[e * 8 + s] = (float)(0.5 * det / (J0[s] * J0[s]));
-          if (c->cplx && (terms_mask & FE_KS_TERM_K)) cell_coef[e * 8 + 4 + s] = (float)(kp[s] * det / J0[s]);
+          if (terms_mask & FE_KS_TERM_T) put(s, 0.5 * det / (J0[s] * J0[s]));
+          if (c->cplx && (terms_mask & FE_KS_TERM_K)) put(4 + s, kp[s] * det / J0[s]);
         }
       }
     }
@@ -467,8 +471,10 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
   {
     std::vector<int> cnt(m, 0);
     for (int64_t i = 0; i < E * np3; ++i) ++cnt[prob->cell_dofs[i]];
-    int64_t slots = 0;
-    for (int64_t d = 0; d < m; ++d) {
+    int64_t slots = 0, shared = 0;
+    for (int64_t d = 0; d < m; ++d) shared += cnt[d] > 1 ? cnt[d] : 0;
+    if (shared > INT32_MAX / 2) asm_dst.clear();   // slot numbers are 32-bit: colour by colour only
+    for (int64_t d = 0; d < m && !asm_dst.empty(); ++d) {
       if (cnt[d] < 2) {
         cnt[d] = -1;
         continue;
@@ -481,7 +487,7 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
     }
     asm_ptr.push_back((int)slots);
     for (const int e : colour_cells)
-      for (int i = 0; i < np3; ++i) {
+      for (int i = 0; i < np3 && !asm_dst.empty(); ++i) {
         const int d = prob->cell_dofs[(int64_t)e * np3 + i];
         asm_dst[(int64_t)e * np3 + i] = cnt[d] < 0 ? d : ~cnt[d]++;
       }
@@ -619,17 +625,8 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
       ok = ok && chk(upload(c, &c->tc5_cst16, cst.data(), cst.size()));
     }
   }
-  if (ok) {
-    // slots for as many columns as kAsmBytes holds (all of n_v_max where that is less)
-    const size_t full = (size_t)c->n_wslots * n_v_max * (c->cplx ? 2 : 1) * sizeof(double);
-    c->asm_bytes = std::min(full, kAsmBytes);
-    ok = chk(upload(c, &c->asm_dst, asm_dst.data(), asm_dst.size())) &&
-         chk(upload(c, &c->asm_dof, asm_dof.data(), asm_dof.size())) &&
-         chk(upload(c, &c->asm_ptr, asm_ptr.data(), asm_ptr.size())) &&
-         chk(upload<char>(c, reinterpret_cast<char**>(&c->asm_W), nullptr, c->asm_bytes));
-  }
   if (ok && boxes.load()) {
-    for (int q = 0; q < nq; ++q) c->gauss_w[q] = (float)wg[q];
+    for (int q = 0; q < nq; ++q) c->gauss_w[q] = wg[q];
     ok = chk(upload(c, &c->cell_coef, cell_coef.data(), cell_coef.size()));
   }
   if (ok && want_nl) {
@@ -658,6 +655,19 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
         build_tc_fpack(c->np, c->cplx != 0, prob->n_proj, c->n_pairs, F.data(), 2, fpack);
         ok = chk(upload(c, &c->tc_fpack_lo, fpack.data(), fpack.size()));
       }
+    }
+  }
+  if (ok && !asm_dst.empty()) {
+    // slots for as many columns as kAsmBytes holds (all of n_v_max where that is less); a
+    // device too full for them goes colour by colour
+    const size_t full = (size_t)c->n_wslots * n_v_max * (c->cplx ? 2 : 1) * sizeof(double);
+    c->asm_bytes = std::min(full, kAsmBytes);
+    if (!(chk(upload<char>(c, reinterpret_cast<char**>(&c->asm_W), nullptr, c->asm_bytes)) &&
+          chk(upload(c, &c->asm_dof, asm_dof.data(), asm_dof.size())) &&
+          chk(upload(c, &c->asm_ptr, asm_ptr.data(), asm_ptr.size())) &&
+          chk(upload(c, &c->asm_dst, asm_dst.data(), asm_dst.size())))) {
+      c->asm_dst = nullptr;
+      g_last_error.clear();
     }
   }
   if (!ok) {
@@ -864,7 +874,10 @@ fe_ks_status apply_core(Ctx& c, const T* X, T* Y, int64_t ncols, bool scaled, T 
   lp.tab = od.tab;
   if constexpr (std::is_same<T, float>::value) {
     lp.cell_coef = c.cell_coef;
-    for (int q = 0; q < c.nq; ++q) lp.w[q] = c.gauss_w[q];
+    for (int q = 0; q < c.nq; ++q) {
+      lp.w[q] = (float)c.gauss_w[q];
+      lp.wl[q] = (float)(c.gauss_w[q] - (double)lp.w[q]);
+    }
   }
   const cudaError_t err = launch_cells<T, T>(c, lp, one, !zero_fill, &nlaunch[2], [&]() -> cudaError_t {
     if constexpr (std::is_same<T, float>::value) {

@@ -82,13 +82,14 @@ struct LocalParams {
   T alpha;                 // Y += alpha * (H X) (1 for a plain application)
   // default kernel (fe_ks_line.cuh): one launch for all cells (cells = nullptr,
   // dst: rows met by one cell are stored to Y, shared rows to their slots of W,
-  // summed by launch_assemble); axis-aligned cells (cell_coef: [E][8] scalars of
-  // the kinetic (0..2) and Bloch (4..6) coefficients, w: 1D Gauss weights)
+  // summed by launch_assemble); axis-aligned cells (cell_coef: [E][16] scalars of
+  // the kinetic (0..2) and Bloch (4..6) coefficients, their remainders 8 later;
+  // w, wl: 1D Gauss weights and their remainders)
   const int* dst;
   TS* W;
   int accum;               // one launch: Y += instead of Y =
   const T* cell_coef;
-  T w[kMaxN];
+  T w[kMaxN], wl[kMaxN];
   EOTables<T> tab;
 };
 
@@ -159,7 +160,7 @@ struct Ctx {
   int inject_fault = 0;            // host-side fault injection into the tcgen05 cell kernel (tests)
   // axis-aligned cells (every cell a box): per-cell scalars of the FP32 default kernel, 1D Gauss weights
   float* cell_coef = nullptr;
-  float gauss_w[kMaxN] = {};
+  double gauss_w[kMaxN] = {};
   // one-launch assembly: destination of every cell node (row of Y when one cell
   // meets the DoF, else ~slot of W), the shared DoFs with their slot ranges, and
   // the slots' values

@@ -355,14 +355,21 @@ __global__ void __launch_bounds__(LineShape<NQ, FORM == kLineSmall>::NT, line_bl
         cf = reinterpret_cast<const T*>(cfs) + ln - (BOX ? 6 * NQ3 : 0);
       else
         cf = p.coef + (int64_t)e * p.ncoef * NQ3 + ln;
-      // axis-aligned cells: kinetic and Bloch coefficients are scalars of the cell times the point's weight
-      T c0{}, c1{}, c2{}, k0{}, k1{}, k2{};
+      // axis-aligned cells: kinetic and Bloch coefficients are scalars of the cell times the point's
+      // weight, formed in pairs so that they round once, as the stored ones do
+      [[maybe_unused]] ff2 cs[3] = {}, ks[3] = {};
       if constexpr (BOX) {
-        const T w2 = p.w[ln % NQ] * p.w[ln / NQ];
-        const T* cc = p.cell_coef + 8 * (int64_t)e;
-        c0 = cc[0] * w2, c1 = cc[1] * w2, c2 = cc[2] * w2;
-        if constexpr (CPLX) k0 = cc[4] * w2, k1 = cc[5] * w2, k2 = cc[6] * w2;
+        const ff2 w2 = ff_mul(ff_make(p.w[ln % NQ], p.wl[ln % NQ]), ff_make(p.w[ln / NQ], p.wl[ln / NQ]));
+        const float* cc = p.cell_coef + 16 * (int64_t)e;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          cs[d] = ff_mul(ff_make(cc[d], cc[8 + d]), w2);
+          if constexpr (CPLX) ks[d] = ff_mul(ff_make(cc[4 + d], cc[12 + d]), w2);
+        }
       }
+      [[maybe_unused]] auto weighted = [&](ff2 c, int q) -> float {
+        return fmaf(c.hi, p.w[q], fmaf(c.hi, p.wl[q], c.lo * p.w[q]));
+      };
 #pragma unroll
       for (int q = 0; q < NQ; ++q) {
         const int s = oz + q * SZ;
@@ -370,10 +377,9 @@ __global__ void __launch_bounds__(LineShape<NQ, FORM == kLineSmall>::NT, line_bl
         const V gx = B[s], gy = C[s], gz = g[q], uu = u[q];
         V z = T(cq[6 * NQ3]) * uu, w0, w1, w2;
         if constexpr (BOX) {
-          const T wz = p.w[q];
-          w0 = (c0 * wz) * gx;
-          w1 = (c1 * wz) * gy;
-          w2 = (c2 * wz) * gz;
+          w0 = weighted(cs[0], q) * gx;
+          w1 = weighted(cs[1], q) * gy;
+          w2 = weighted(cs[2], q) * gz;
         } else {
           const T G00 = cq[0], G01 = cq[NQ3], G02 = cq[2 * NQ3], G11 = cq[3 * NQ3], G12 = cq[4 * NQ3];
           const T G22 = cq[5 * NQ3];
@@ -391,8 +397,7 @@ __global__ void __launch_bounds__(LineShape<NQ, FORM == kLineSmall>::NT, line_bl
         if constexpr (CPLX) {
           V kk;
           if constexpr (BOX) {
-            const T wz = p.w[q];
-            kk = wz * fma(k0, gx, fma(k1, gy, k2 * gz));
+            kk = fma(weighted(ks[0], q), gx, fma(weighted(ks[1], q), gy, weighted(ks[2], q) * gz));
           } else {
             kk = fma(T(cq[10 * NQ3]), gx, fma(T(cq[11 * NQ3]), gy, T(cq[12 * NQ3]) * gz));
           }
