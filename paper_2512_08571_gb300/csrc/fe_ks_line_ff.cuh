@@ -65,7 +65,7 @@ struct LineShapeFF {
 
 template <int NP, int NQ, bool CPLX, bool SMALL>
 __global__ void __launch_bounds__(LineShapeFF<NQ, SMALL>::NT, LineShapeFF<NQ, SMALL>::MINB)
-    fe_line_ff_kernel(const __grid_constant__ LocalParams<ff2, double> p) {
+    fe_line_ff_kernel(const __grid_constant__ LocalParams<ff2, double> p, int per_sm) {
   using S = LineShapeFF<NQ, SMALL>;
   using E = Elem<ff2, double>;
   constexpr int VG = S::VG, SX = S::SX, SY = S::SY, SZ = S::SZ, NQ2 = NQ * NQ, NQ3 = NQ * NQ2, NP2 = NP * NP;
@@ -78,7 +78,14 @@ __global__ void __launch_bounds__(LineShapeFF<NQ, SMALL>::NT, LineShapeFF<NQ, SM
   const int64_t ntiles = (nslots + VG - 1) / VG;
   const bool gauss_line = ln < NQ2;
   const unsigned gmask = CPLX ? __ballot_sync(0xffffffffu, gauss_line) : 0u;
-  for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+  // In full rounds the blocks that share a multiprocessor (b, b + sms, ...) take neighbouring tiles, so
+  // that its L1 serves a cell's coefficients to them (8^3 cells, p = 8, 64 columns: 1770 -> 1697 us);
+  // the last round spreads over the multiprocessors.
+  const int sms = gridDim.x / per_sm, near = (int)(blockIdx.x % sms) * per_sm + (int)(blockIdx.x / sms);
+  const int64_t full = ntiles / gridDim.x * gridDim.x;
+  for (int64_t r = 0; r < ntiles; r += gridDim.x) {
+    const int64_t t = r + (r < full ? near : (int)blockIdx.x);
+    if (t >= ntiles) break;
     // an idle lane repeats a slot of its own re/im parity and stores nothing
     const int64_t slot = t * VG + v;
     const bool act = slot < nslots;
@@ -252,7 +259,7 @@ cudaError_t launch_line_ff_form(const Ctx& c, const LocalParams<ff2, double>& pr
     attr_done[dev] = true;
   }
   const int64_t ntiles = ((int64_t)prm.n_cells * prm.ncols + S::VG - 1) / S::VG, slots = (int64_t)S::MINB * sms;
-  k<<<(int)(ntiles < slots ? ntiles : slots), S::NT, S::bytes, s>>>(prm);
+  k<<<(int)(ntiles < slots ? ntiles : slots), S::NT, S::bytes, s>>>(prm, ntiles < slots ? 1 : S::MINB);
   return cudaGetLastError();
 }
 
