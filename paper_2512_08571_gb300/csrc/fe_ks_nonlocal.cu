@@ -149,6 +149,16 @@ __device__ __forceinline__ void ld16(const ff2* p, ff2* o) {
   o[0] = ff_make(v.x, v.y), o[1] = ff_make(v.z, v.w);
 }
 
+__device__ __forceinline__ void st16(float* p, const float* v) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void st16(double* p, const double* v) {
+  *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+}
+__device__ __forceinline__ void st16(ff2* p, const ff2* v) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0].hi, v[0].lo, v[1].hi, v[1].lo);
+}
+
 // Elements per node of the transposed F block: MAXP projectors (x2 complex),
 // rounded up to a whole number of 16-byte chunks.
 template <typename TF, bool CPLX, int MAXP>
@@ -182,11 +192,17 @@ fe_proj_pair_kernel(const TS* __restrict__ Xg, int64_t ld, int ncols, const int*
   const int c0 = (blockIdx.y * cg + lc) * V;
   const bool vec = (ld % V == 0) && (((uintptr_t)Xg & 15) == 0) && c0 + V <= ncols;
   const TF* Fp = Fg + (int64_t)pr * nf;
-  // transpose F[b][node][re,im] -> Fs[node][b][re,im] (global reads coalesced over node)
-  for (int i = threadIdx.x; i < nf; i += kPairThreads) {
-    const int b = i / (np3 * CW), rem = i - b * np3 * CW;
-    const int node = rem / CW, ri = rem - node * CW;
-    Fs[node * PB + b * CW + ri] = Fp[i];
+  // transpose F[b][node][re,im] -> Fs[node][b][re,im]: a node per thread, all its projectors in flight
+  // (coalesced over the nodes), 16-byte shared stores
+  for (int node = threadIdx.x; node < np3; node += kPairThreads) {
+    TF row[PB];
+#pragma unroll
+    for (int q = 0; q < PB; ++q) {
+      const int b = q / CW;
+      row[q] = b < n_proj ? Fp[((int64_t)b * np3 + node) * CW + q % CW] : TF{};
+    }
+#pragma unroll
+    for (int q = 0; q < PB; q += 16 / (int)sizeof(TF)) st16(Fs + node * PB + q, row + q);
   }
   const int cell = pair_cell[pr];
   for (int i = threadIdx.x; i < np3; i += kPairThreads) ds[i] = cell_dofs[(int64_t)cell * np3 + i];
