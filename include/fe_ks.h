@@ -155,7 +155,8 @@ fe_ks_status fe_ks_quadrature_points(const fe_ks_problem* prob, double* xq_out);
  * coefficients (Sec. 3.1 eq. reformcellmat with the Jacobian scaling folded
  * in), cell-level projector matrices F^(a,e) (eq. Vnonloc), a conflict-free
  * colouring of the cells for the scatter-add, the GLL-lumped mass D, and all
- * device workspace for n_v_max vectors.  terms_mask selects the terms of H.
+ * device workspace for n_v_max vectors (up to 256 MiB of it assembly slots, one
+ * per cell node on a shared DoF and column).  terms_mask selects the terms of H.
  * cuda_stream (cudaStream_t, may be NULL = legacy default stream) orders all
  * later calls.  Returns FE_KS_ERR_MESH for out-of-range DoFs or det J <= 0.
  */
@@ -256,7 +257,12 @@ fe_ks_status fe_ks_cheb_filter_ghep(fe_ks_ctx* ctx, fe_ks_ctx* mass, double* X, 
  * direction).  Complex operators and FE_KS_BF16X2 have the warp-level kernel
  * only.  FE_KS_F64, FE_KS_F32,
  * FE_KS_F64E:
- *   0..2  one CTA per (cell, column tile), 3 tile widths;
+ *   0     fused line sweeps over tiles of (cell, column) pairs, the form chosen by
+ *         shape: a block per cell with its tables in shared memory (FP32, a tile
+ *         of columns or more), flattened tiles otherwise, small ones for small
+ *         problems; all cells in one launch where the context's assembly slots
+ *         hold the columns, else a launch per colour (same bits);
+ *   1..2  one CTA per (cell, column tile), 2 tile widths;
  *   3..4  one CTA per cell walking all column tiles, the next tile's rows of X
  *         staged by cp.async, reduction-based scatter;
  *   5..6  as 3..4 with 2 or 4 adjacent columns per thread;
@@ -361,9 +367,10 @@ fe_ks_status fe_ks_colour_cells(int64_t n_cells, int32_t np3, int64_t n_dofs, co
  * Batched application: Y_s = H_s X_s for up to 16 independent systems of
  * uneven size, degree, vector count and precision in ONE call.  Real FP64 /
  * FP32 systems of degree 4..8 with n_q = n_p go to ONE persistent kernel
- * launch: the work queue is phase-major -- zero-fill of every Y_s and the
- * per-atom projections first, then the cells of colour 0, 1, ... of every
- * system -- and a work item of system s waits (bounded) for the completion of
+ * launch: the work queue is phase-major -- the per-atom projections first, then
+ * every cell and the sums of the shared rows (systems with projectors whose
+ * assembly slots hold the columns), or zero-fill of Y_s and the cells of
+ * colour 0, 1, ... (the others) -- and a work item of system s waits (bounded) for the completion of
  * s's previous phase only, so systems overlap freely.  Every other system
  * (complex operators, n_q = n_p + 2, degrees 1..3, FE_KS_F64E / FE_KS_BF16 /
  * FE_KS_F16 / FE_KS_BF16X2) is a direct system (fe_ks_batch_set_direct below):
