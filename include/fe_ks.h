@@ -255,8 +255,9 @@ fe_ks_status fe_ks_cheb_filter_ghep(fe_ks_ctx* ctx, fe_ks_ctx* mass, double* X, 
  * one's first plane product (0, the default), at once (2) or after its first
  * quadrature-point step (3); 1 = the warp-level MMA kernel (one sweep per
  * direction).  Complex operators and FE_KS_BF16X2 have the warp-level kernel
- * only.  FE_KS_F64, FE_KS_F32,
- * FE_KS_F64E:
+ * only.  All of them run every cell in one launch where the context's assembly
+ * slots hold the columns, else a launch per colour (same bits).  FE_KS_F64,
+ * FE_KS_F32, FE_KS_F64E:
  *   0     fused line sweeps over tiles of (cell, column) pairs, the form chosen by
  *         shape: a block per cell with its tables in shared memory (FP32, a tile
  *         of columns or more), flattened tiles otherwise, small ones for small

@@ -755,11 +755,14 @@ fe_ks_status fe_ks_info(const fe_ks_ctx* ctx, int64_t* n_dofs, int64_t* n_cells,
 
 namespace feks {
 
-// Whether this application may go through the context's slots: the default kernel, slots
-// large enough, and nobody else in them.  An operator with projectors has per-context
-// scratch anyway (Q and its partials), so its applications are ordered by the caller; one
-// without has none, and may run on several streams at once: only its set-up stream, and no
-// graph captured there, takes the slots, every other application goes colour by colour.
+// Whether this application may go through the context's slots: the default kernel (cfg 0) or a
+// tensor-core one, slots large enough, and nobody else in them.  An operator with projectors
+// has per-context scratch anyway (Q and its partials), so its applications are ordered by the
+// caller; one without has none, and may run on several streams at once: only its set-up
+// stream, and no graph captured there, takes the slots, every other application goes colour
+// by colour.  Tensor-core kernels, by colour -> one launch: FP16 p = 6, 8^3 cells, 64 columns
+// 288 -> 173 us; FP16 p = 3, 12^3, 16 columns 144 -> 91 us; BF16x2 p = 8, 8^3, 64 columns
+// 741 -> 637 us; complex BF16 p = 7, 8^3, 24 columns 268 -> 185 us.
 static bool one_launch(const Ctx& c, int cfg, int64_t ncols, size_t esize) {
   if (cfg != 0 || !asm_fits(c, ncols, esize)) return false;
   if ((c.terms & FE_KS_TERM_NL) && c.n_pairs > 0) return true;
@@ -824,7 +827,7 @@ fe_ks_status apply_core(Ctx& c, const T* X, T* Y, int64_t ncols, bool scaled, T 
     c.ev_pool.pop_back();
     cudaEventRecord(ev[i], s);
   };
-  const bool one = !tc && one_launch(c, sizeof(T) == 8 ? c.cfg64 : c.cfg32, ncols, sizeof(T));
+  const bool one = one_launch(c, tc ? 0 : sizeof(T) == 8 ? c.cfg64 : c.cfg32, ncols, sizeof(T));
   mark(0);
   if (zero_fill && !one && cudaMemsetAsync(Y, 0, bytes, s) != cudaSuccess)
     return fail(FE_KS_ERR_CUDA, "cudaMemsetAsync failed");

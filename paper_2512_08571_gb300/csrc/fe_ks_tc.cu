@@ -47,6 +47,9 @@ struct TcParams {
   const int* cell_dofs;
   const int* cells;
   int n_cells;
+  const int* dst;      // one launch for all cells: row of Y, or ~slot of W, per cell node; else nullptr
+  float* W;
+  int accum;           // one launch: Y += instead of Y =
   const float* coef;       // [E][ncoef][n^3]
   int ncoef;
   int gga;
@@ -325,10 +328,11 @@ __device__ __forceinline__ float tile_scale(float mx) {
 // Assembly Y += alpha D^{-1/2} Q^T Y^(e) of the staged FP32 cell result for
 // columns [c0, c0 + 8): one node per thread, two 16-byte reductions per node
 // when the rows are 16-byte aligned.  Colour-exclusive launches: no other
-// cell of the launch touches the same DoF rows.
+// cell of the launch touches the same DoF rows.  One launch for all cells (dst):
+// plain stores to Y or to the node's slot.
 template <int N, bool CPLX, bool F16>
-__device__ __forceinline__ void scatter_stage(const TcParams& p, const float* stage, const int* sd, int c0, bool vecy,
-                                              const float* unscale) {
+__device__ __forceinline__ void scatter_stage(const TcParams& p, const float* stage, const int* sd, int e, int c0,
+                                              bool vecy, const float* unscale) {
   using Gm = Geom<N, CPLX>;
   const bool fullv = vecy && c0 + 8 <= p.ncols;
   float4 ua = make_float4(1.f, 1.f, 1.f, 1.f), ub = ua;   // per-column unscale (FP16)
@@ -344,6 +348,27 @@ __device__ __forceinline__ void scatter_stage(const TcParams& p, const float* st
     const float sc = p.dscale ? p.alpha * __ldg(p.dscale + d) : p.alpha;
     a.x *= sc * ua.x, a.y *= sc * ua.y, a.z *= sc * ua.z, a.w *= sc * ua.w;
     b.x *= sc * ub.x, b.y *= sc * ub.y, b.z *= sc * ub.z, b.w *= sc * ub.w;
+    if (p.dst) {   // one launch for all cells: rows of one cell straight to Y, shared rows to their slots
+      const int q = __ldg(p.dst + (int64_t)e * Gm::N3 + node);
+      float* yp = q >= 0 ? p.Y + (int64_t)q * p.ld + c0 : p.W + (int64_t)(~q) * p.ld + c0;
+      const bool add = p.accum && q >= 0;
+      if (fullv) {
+        float4* y4 = reinterpret_cast<float4*>(yp);
+        if (add) {
+          const float4 oa = y4[0], ob = y4[1];
+          a.x += oa.x, a.y += oa.y, a.z += oa.z, a.w += oa.w;
+          b.x += ob.x, b.y += ob.y, b.z += ob.z, b.w += ob.w;
+        }
+        y4[0] = a;
+        y4[1] = b;
+      } else {
+        const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          if (c0 + c < p.ncols) yp[c] = add ? yp[c] + v[c] : v[c];
+      }
+      continue;
+    }
     float* yp = p.Y + (int64_t)d * p.ld + c0;
     if (fullv) {
       atomicAdd(reinterpret_cast<float4*>(yp), a);
@@ -403,7 +428,7 @@ __global__ void __launch_bounds__(Geom<N, CPLX, SPLIT>::NT, Geom<N, CPLX, SPLIT>
   const bool vecy = (p.ld % 4 == 0) && (((uintptr_t)p.Y & 15) == 0);
 
   for (int ci = blockIdx.x; ci < p.n_cells; ci += gridDim.x) {
-    const int e = p.cells[ci];
+    const int e = p.cells ? p.cells[ci] : ci;
     __syncthreads();   // the previous cell's scatter has finished with sd
     // stage the DoF list and the coefficients, point-major [pt][NC]
     for (int w = tid; w < N3; w += NT) sd[w] = p.cell_dofs[(int64_t)e * N3 + w];
@@ -455,7 +480,7 @@ __global__ void __launch_bounds__(Geom<N, CPLX, SPLIT>::NT, Geom<N, CPLX, SPLIT>
             if (p.dscale) sc[r] = __ldg(p.dscale + d);
           }
         }
-        if (prev0 >= 0) scatter_stage<N, CPLX, F16>(p, stage, sd, prev0, vecy, unscale);
+        if (prev0 >= 0) scatter_stage<N, CPLX, F16>(p, stage, sd, e, prev0, vecy, unscale);
         // FP16: scale every column of the tile by a power of two so that its
         // largest entry is below 1/16 (exact; undone at the scatter)
         float cs[8] = {1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f};
@@ -838,7 +863,7 @@ __global__ void __launch_bounds__(Geom<N, CPLX, SPLIT>::NT, Geom<N, CPLX, SPLIT>
       __syncthreads();   // the stage is complete; array 2 is free for the next extraction
       prev0 = col0;
     }
-    if (prev0 >= 0) scatter_stage<N, CPLX, F16>(p, stage, sd, prev0, vecy, unscale);
+    if (prev0 >= 0) scatter_stage<N, CPLX, F16>(p, stage, sd, e, prev0, vecy, unscale);
   }
 }
 
@@ -923,6 +948,9 @@ cudaError_t launch_tc(const Ctx& c, const LocalParams<float>& lp, cudaStream_t s
   p.cell_dofs = lp.cell_dofs;
   p.cells = lp.cells;
   p.n_cells = lp.n_cells;
+  p.dst = lp.dst;
+  p.W = lp.W;
+  p.accum = lp.accum;
   p.coef = lp.coef;
   p.ncoef = lp.ncoef;
   p.gga = lp.gga;

@@ -266,8 +266,11 @@ struct Params {
   int64_t ld;
   int ncols;
   const int* cell_dofs;
-  const int* cells;
+  const int* cells;      // cells of the launch (nullptr: all, in order)
   int n_cells;
+  const int* dst;        // one launch for all cells: row of Y, or ~slot of W, per cell node; else nullptr
+  float* W;
+  int accum;             // one launch: Y += instead of Y =
   const float* coef;     // [E][ncoef][N^3]
   int ncoef;
   int gga;
@@ -457,7 +460,7 @@ __global__ void __launch_bounds__(512, 1) fe_tc5_kernel(const __grid_constant__ 
     const int t_begin = (u % p.units_per_cell) * p.tiles_per_unit;
     const int t_end = min(ntiles, t_begin + p.tiles_per_unit);
     if (t_begin >= t_end) continue;
-    const int e = p.cells[ci];
+    const int e = p.cells ? p.cells[ci] : ci;
     __syncthreads();   // both pipelines have finished the previous unit
     if (ci != staged) {
       for (int w = tid; w < N3; w += NT) {
@@ -865,6 +868,24 @@ __global__ void __launch_bounds__(512, 1) fe_tc5_kernel(const __grid_constant__ 
             float w[VT];
 #pragma unroll
             for (int v = 0; v < VT; ++v) w[v] = s * fmaf(o[j][v], usc[ub * VT + v], ex[j][v]);
+            if (p.dst) {   // rows of one cell straight to Y, shared rows to their slots
+              const int q = __ldg(p.dst + (int64_t)e * N3 + pp + NN * c);
+              float* yp = q >= 0 ? p.Y + (int64_t)q * p.ld + col0 : p.W + (int64_t)(~q) * p.ld + col0;
+              const bool add = p.accum && q >= 0;
+              if (vecy && col0 + VT <= p.ncols) {
+                float4 r = make_float4(w[0], w[1], w[2], w[3]);
+                if (add) {
+                  const float4 o4 = *reinterpret_cast<const float4*>(yp);
+                  r.x += o4.x, r.y += o4.y, r.z += o4.z, r.w += o4.w;
+                }
+                *reinterpret_cast<float4*>(yp) = r;
+              } else {
+#pragma unroll
+                for (int v = 0; v < VT; ++v)
+                  if (col0 + v < p.ncols) yp[v] = add ? yp[v] + w[v] : w[v];
+              }
+              continue;
+            }
             float* yp = p.Y + (int64_t)d * p.ld + col0;
             if (vecy && col0 + VT <= p.ncols) {
               atomicAdd(reinterpret_cast<float4*>(yp), make_float4(w[0], w[1], w[2], w[3]));
@@ -1011,6 +1032,9 @@ cudaError_t launch_tc5(const Ctx& c, const LocalParams<float>& lp, cudaStream_t 
   p.cell_dofs = lp.cell_dofs;
   p.cells = lp.cells;
   p.n_cells = lp.n_cells;
+  p.dst = lp.dst;
+  p.W = lp.W;
+  p.accum = lp.accum;
   p.coef = lp.coef;
   p.ncoef = lp.ncoef;
   p.gga = lp.gga;

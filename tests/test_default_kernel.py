@@ -22,7 +22,7 @@ from paper_2512_08571_gb300 import fe_ks as fk
 from synth.host_problem import HostProblem
 from oracle.operator import Problem
 from synth import Workload, trial_vectors
-from gpu_util import gpu_apply, parity_err, round_input
+from gpu_util import gpu_apply, parity_err, round_input, torch_dtype
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -99,14 +99,17 @@ def test_same_bits_twice(precision):
     assert np.array_equal(a, b)
 
 
-@pytest.mark.parametrize("precision", PREC)
-def test_one_launch_gives_the_bits_of_the_colour_launches(precision):
+TC = (fk.FE_KS_BF16, fk.FE_KS_F16, fk.FE_KS_BF16X2)
+
+
+@pytest.mark.parametrize("precision,p,cplx,nv", [(q, 5, False, 13) for q in PREC] + [
+    (q, p, cplx, nv) for q in TC for p in (3, 8) for cplx in (False, True) for nv in (13, 24)])
+def test_one_launch_gives_the_bits_of_the_colour_launches(precision, p, cplx, nv):
     """Operator without projectors: the set-up stream takes the one-launch assembly, another
     stream and a captured graph go colour by colour; all the same bits."""
-    wl = _wl(5, False, 0.05, n=3, n_atoms=0, n_v=13)
+    wl = _wl(p, cplx, 0.05, n=3, n_atoms=0, n_v=nv)
     hp = HostProblem(wl)
-    dt = torch.float32 if precision == fk.FE_KS_F32 else torch.float64
-    X = torch.from_numpy(trial_vectors(wl)).cuda().to(dt)
+    X = torch.from_numpy(trial_vectors(wl)).cuda().to(torch_dtype(precision, cplx))
     ys = [torch.full_like(X, float("nan")) for _ in range(3)]
     side = torch.cuda.Stream()
     home = torch.cuda.Stream()
