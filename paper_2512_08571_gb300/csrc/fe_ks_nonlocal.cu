@@ -134,6 +134,15 @@ cudaError_t launch_proj_emu(const Ctx& c, const ProjParams<double>& prm, const f
 // ---- pair form
 
 constexpr int kPairThreads = 256;
+// Blocks per SM of the pair kernel (a register cap of 80 or 128): the gather is bound by the
+// latency of its rows, so blocks count more than a few spilled values.  Real, up to 9
+// projectors, 3 blocks / 2 at 959 pairs, p = 6, 64 FP64 columns: 411 / 458 us; 782 pairs, p = 8,
+// 1 column in pairs of floats: 33 / 39 us.  Four (64 registers) spill: FP32, 1883 pairs, p = 8,
+// 256 columns 320 -> 342 us.
+template <typename T, bool CPLX, int MAXP>
+constexpr int pair_blocks() {
+  return MAXP <= 9 ? (CPLX && std::is_same<T, ff2>::value ? 2 : 3) : std::is_same<T, double>::value && !CPLX ? 1 : 2;
+}
 
 // 16 bytes of shared memory into 16 / sizeof(TF) values (one vector load)
 __device__ __forceinline__ void ld16(const float* p, float* o) {
@@ -169,11 +178,11 @@ __host__ __device__ constexpr int pair_fstride() {
 // P[pr][b][col] = sum_node conj(F[pr][b][node]) x(d(node), col), x scaled by
 // D^{-1/2} when dscale is given.  Each thread owns V = 16 / sizeof(TS)
 // adjacent columns (one 16-byte load per row; for complex data the re/im
-// partner is in the same thread); cg (a power of two) column groups per CTA, the
-// 256 / cg row slices of a CTA reduced within each warp by shuffles (cg < 32) and
-// then in shared memory in slice order.  MAXP >= n_proj.
+// partner is in the same thread); cg column groups per CTA, the 256 / cg row
+// slices of a CTA reduced within each warp by shuffles (cg a power of two below
+// 32) and then in shared memory (over F) in slice order.  MAXP >= n_proj.
 template <typename T, typename TS, typename TF, bool CPLX, int MAXP>
-__global__ void __launch_bounds__(kPairThreads)
+__global__ void __launch_bounds__(kPairThreads, (pair_blocks<T, CPLX, MAXP>()))
 fe_proj_pair_kernel(const TS* __restrict__ Xg, int64_t ld, int ncols, const int* __restrict__ cell_dofs,
                     const int* __restrict__ pair_cell, const TF* __restrict__ Fg, const TS* __restrict__ dscale,
                     TS* __restrict__ part, int n_proj, int np3, int cg) {
@@ -185,7 +194,7 @@ fe_proj_pair_kernel(const TS* __restrict__ Xg, int64_t ld, int ncols, const int*
   TF* Fs = reinterpret_cast<TF*>(smp);   // [node][PB]
   const int nf = n_proj * np3 * CW;
   int* ds = reinterpret_cast<int*>(smp + (size_t)np3 * PB * sizeof(TF));
-  T* red = reinterpret_cast<T*>(smp + (((size_t)np3 * PB * sizeof(TF) + (size_t)np3 * sizeof(int) + 15) & ~(size_t)15));
+  T* red = reinterpret_cast<T*>(smp);    // over Fs, once every row is done
   const int pr = blockIdx.x;
   const int rs = kPairThreads / cg;
   const int lc = threadIdx.x % cg, sl = threadIdx.x / cg;
@@ -213,7 +222,7 @@ fe_proj_pair_kernel(const TS* __restrict__ Xg, int64_t ld, int ncols, const int*
 #pragma unroll
     for (int v = 0; v < V; ++v) acc[b][v] = N::zero();
   constexpr int RU = 4;   // rows in flight per thread
-  for (int n0 = sl; n0 < np3; n0 += RU * rs) {
+  for (int n0 = sl < rs ? sl : np3; n0 < np3; n0 += RU * rs) {
     TS xs[RU][V];
 #pragma unroll
     for (int u = 0; u < RU; ++u) {
@@ -272,13 +281,16 @@ fe_proj_pair_kernel(const TS* __restrict__ Xg, int64_t ld, int ncols, const int*
     }
   }
   // fewer than 32 groups: the warp's row slices, in a fixed tree
-  for (int o = 16; o >= cg; o >>= 1)
+  const bool tree = cg < 32 && (cg & (cg - 1)) == 0;
+  if (tree)
+    for (int o = 16; o >= cg; o >>= 1)
 #pragma unroll
-    for (int b = 0; b < MAXP; ++b)
-      if (b < n_proj)
+      for (int b = 0; b < MAXP; ++b)
+        if (b < n_proj)
 #pragma unroll
-        for (int v = 0; v < V; ++v) acc[b][v] = acc[b][v] + N::shfl_xor(acc[b][v], o);
+          for (int v = 0; v < V; ++v) acc[b][v] = acc[b][v] + N::shfl_xor(acc[b][v], o);
   if (rs == 1) {
+    if (sl > 0) return;
 #pragma unroll
     for (int b = 0; b < MAXP; ++b)
       if (b < n_proj)
@@ -288,8 +300,9 @@ fe_proj_pair_kernel(const TS* __restrict__ Xg, int64_t ld, int ncols, const int*
     return;
   }
   const int cols = cg * V;   // columns of this CTA
-  const int ns = cg < 32 ? kPairThreads / 32 : rs, row = cg < 32 ? threadIdx.x / 32 : sl;   // partial sums left
-  if (cg >= 32 || (threadIdx.x & 31) < cg)
+  const int ns = tree ? kPairThreads / 32 : rs, row = tree ? threadIdx.x / 32 : sl;   // partial sums left
+  __syncthreads();           // red lies over Fs
+  if (tree ? (threadIdx.x & 31) < cg : sl < rs)
 #pragma unroll
     for (int b = 0; b < MAXP; ++b)
       if (b < n_proj)
@@ -335,16 +348,16 @@ __global__ void fe_proj_sum_kernel(const TS* __restrict__ part, const TS* __rest
   }
 }
 
-// Column groups (of 16 / sizeof(TS) columns) per CTA of the pair kernel: the
-// smallest power of two covering the columns, at most 256.  With fewer groups
-// than lanes the lanes of a warp take different rows (one column in pairs of
-// floats, 782 pairs at p = 8: 413 us when a group of columns filled a warp).
+// Column groups (of 16 / sizeof(TS) columns) per CTA of the pair kernel, at most 256.  With
+// fewer groups than lanes the lanes of a warp take different rows (one column in pairs of
+// floats, 782 pairs at p = 8: 413 us when a group of columns filled a warp).  Up to four
+// groups: a power of two, the slices of a warp summed by shuffles; above, exactly the
+// columns' groups, so that no lane is without a column (48 columns at p = 6, 485 pairs: FP32, 12
+// groups, 28 us rounded up to 16 and 23 as they are; in pairs of floats, 24 groups, 138 and 87 us).
 template <typename TS>
 static int pair_groups(int ncols) {
   const int groups = (ncols + (16 / (int)sizeof(TS)) - 1) / (16 / (int)sizeof(TS));
-  int cg = 1;
-  while (cg < 256 && cg < groups) cg *= 2;
-  return cg;
+  return groups == 3 ? 4 : std::min(groups, 256);
 }
 
 template <typename T, typename TS, typename TF, bool CPLX, int MAXP>
@@ -354,7 +367,7 @@ static cudaError_t launch_pair_p(const ProjParams<TS>& prm, const TF* F, int n_a
   const int rs = kPairThreads / cg;   // row slices
   constexpr int PB = pair_fstride<TF, CPLX, MAXP>();
   const size_t head = ((size_t)prm.np3 * PB * sizeof(TF) + (size_t)prm.np3 * sizeof(int) + 15) & ~(size_t)15;
-  const size_t smem = head + (rs > 1 ? (size_t)std::min(rs, cg < 32 ? kPairThreads / 32 : rs) * prm.n_proj * cg * V * sizeof(T) : 0);
+  const size_t smem = std::max(head, rs > 1 ? (size_t)rs * prm.n_proj * cg * V * sizeof(T) : 0);   // sums over F
   if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
   cudaError_t err = cudaFuncSetAttribute(fe_proj_pair_kernel<T, TS, TF, CPLX, MAXP>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

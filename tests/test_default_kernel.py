@@ -132,3 +132,18 @@ def test_one_launch_gives_the_bits_of_the_colour_launches(precision, p, cplx, nv
         fk.fe_ks_destroy(ctx)
     assert not torch.isnan(ys[0]).any()
     assert torch.equal(ys[0], ys[1]) and torch.equal(ys[0], ys[2])
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("precision", PREC)
+def test_projection_column_groups(precision, cplx):
+    """Column counts around the pair projection's splits of a block: 1, 3, 5, 12, 16, 33, 86, 129 and
+    257 groups of 16 bytes, a column short of whole groups and not."""
+    cols = 16 // (4 if precision == fk.FE_KS_F32 else 8) / (2 if cplx else 1)
+    nvs = sorted({max(1, int(g * cols) - d) for g in (1, 3, 5, 12, 16, 33, 86, 129, 257) for d in (0, 1)})
+    wl = _wl(2, cplx, 0.05, n=3, n_v=max(nvs))
+    hp, X = HostProblem(wl), round_input(trial_vectors(wl), precision)
+    ref = Problem(wl).apply(X)
+    for nv in nvs:
+        Y = gpu_apply(hp, np.ascontiguousarray(X[:, :nv]), precision)
+        assert parity_err(Y, ref[:, :nv]) <= TOL[precision], nv
