@@ -29,6 +29,17 @@
 // that carry projectors are neighbours, and a contiguous share of them would make
 // some blocks late.
 //
+// What bounds it.  FP64: the FP64 pipe (p = 6, 10^3 cells, 64 columns: 0.75 of 1.25 TFLOP/s,
+// 5.15 -> 4.92 ms).  FP32: barriers and the latency of the shared-memory sweeps (p = 8:
+// issue 54 % and FMA pipe 40 % busy with the 32 % of the warps that the three tiles and the staged tables
+// leave room for); keeping lines in registers instead (a plane per thread, 12 accesses a point) takes
+// 8 to 12 thousand straight-line instructions and was bound by the instruction cache, 11.8 ms
+// against 6.4 of the kernels in fe_ks_local.cuh.  By colour there -> here: p = 8, 16^3 cells, 256
+// columns, 19 atoms 7.6 -> 6.6 ms; complex p = 7, 10^3, 64 columns 1.70 -> 0.65 ms; n_q = 11, 8^3,
+// 32 columns 565 -> 235 us; p = 6, 12^3, 37 columns 706 -> 333 us; FP64 p = 4, 4^3, 8 columns
+// 223 -> 24.6 us.  Wide / flat form at p = 8, 16^3, 256
+// columns without atoms: 5.3 / 5.7 ms.
+//
 // Elements: every type works on 8-byte elements -- two FP32 columns (packed FP32x2
 // instructions; the re and im columns of a complex vector), one FP64 column, or
 // one column in a pair of floats (fe_ks_line_ff.cuh).

