@@ -266,7 +266,7 @@ struct Params {
   int64_t ld;
   int ncols;
   const int* cell_dofs;
-  const int* cells;      // cells of the launch (nullptr: all, in order)
+  const int* cells;      // cells of the launch (with dst: all, in order)
   int n_cells;
   const int* dst;        // one launch for all cells: row of Y, or ~slot of W, per cell node; else nullptr
   float* W;
@@ -311,7 +311,9 @@ __device__ __forceinline__ int wait_limit(const Params& p) { return p.inject ? k
 __device__ __forceinline__ void stagger_arrive() { asm volatile("bar.arrive 3, 512;\n" ::: "memory"); }
 __device__ __forceinline__ void stagger_wait() { asm volatile("bar.sync 3, 512;\n" ::: "memory"); }
 
-template <int N, bool F16>
+// ONE: one launch for all cells (p.dst), a variant of its own: as a run-time branch of the scatter it
+// cost the launches by colour 2 to 3 % (FP16, 20^3 cells, p = 8, 256 columns 15.4 / 14.9 ms)
+template <int N, bool F16, bool ONE>
 __global__ void __launch_bounds__(512, 1) fe_tc5_kernel(const __grid_constant__ Params p) {
   using G = G5<N>;
   constexpr int NT = G::NT, GT = G::GT, NN = G::NN, N3 = G::N3, VT = G::VT;
@@ -460,7 +462,7 @@ __global__ void __launch_bounds__(512, 1) fe_tc5_kernel(const __grid_constant__ 
     const int t_begin = (u % p.units_per_cell) * p.tiles_per_unit;
     const int t_end = min(ntiles, t_begin + p.tiles_per_unit);
     if (t_begin >= t_end) continue;
-    const int e = p.cells ? p.cells[ci] : ci;
+    const int e = ONE ? ci : p.cells[ci];
     __syncthreads();   // both pipelines have finished the previous unit
     if (ci != staged) {
       for (int w = tid; w < N3; w += NT) {
@@ -868,7 +870,7 @@ __global__ void __launch_bounds__(512, 1) fe_tc5_kernel(const __grid_constant__ 
             float w[VT];
 #pragma unroll
             for (int v = 0; v < VT; ++v) w[v] = s * fmaf(o[j][v], usc[ub * VT + v], ex[j][v]);
-            if (p.dst) {   // rows of one cell straight to Y, shared rows to their slots
+            if constexpr (ONE) {   // rows of one cell straight to Y, shared rows to their slots
               const int q = __ldg(p.dst + (int64_t)e * N3 + pp + NN * c);
               float* yp = q >= 0 ? p.Y + (int64_t)q * p.ld + col0 : p.W + (int64_t)(~q) * p.ld + col0;
               const bool add = p.accum && q >= 0;
@@ -961,18 +963,29 @@ cudaError_t launch_n(Params p, cudaStream_t s) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (sms <= 0) sms = 152;
-  cudaError_t err = cudaFuncSetAttribute(fe_tc5_kernel<N, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::BYTES);
+  auto kernel = p.dst ? fe_tc5_kernel<N, F16, true> : fe_tc5_kernel<N, F16, false>;
+  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, G::BYTES);
   if (err != cudaSuccess) return err;
   const int ntiles = (p.ncols + G::VT - 1) / G::VT;
   // units of column tiles of one cell: even (the tiles alternate between the CTA's two pipelines),
-  // a unit's start (coefficients, first gather and plane product, drained pipelines) costing
-  // about three tiles: 12^3 cells (216 a colour), p = 8, 256 columns 3.95 ms in about sixteen
-  // units an SM, 3.43 ms in these
-  p.tiles_per_unit = tiles_per_unit(p.n_cells, ntiles, sms, 3.0, 2);
+  // about 16 or more per SM, so that the cells with projectors, which take longer, spread; but the
+  // run with the fewest rounds where that saves an eighth, a unit's start (coefficients, first gather
+  // and plane product, drained pipelines) costing about three tiles.  p = 8, 256 columns: 12^3 cells
+  // (216 a colour) 3.95 ms in 16 units per SM, 3.41 in the fewest rounds; 20^3, 32 atoms 13.7 and 14.4.
+  int upc = 1;
+  while (2 * upc < ntiles && (int64_t)p.n_cells * upc < 16LL * sms) upc *= 2;
+  int run = (ntiles + upc - 1) / upc;
+  run += run & 1;
+  auto cost = [&](int r) {
+    const int64_t units = (int64_t)p.n_cells * ((ntiles + r - 1) / r);
+    return (double)((units + sms - 1) / sms) * (r + 3.0);
+  };
+  const int few = tiles_per_unit(p.n_cells, ntiles, sms, 3.0, 2);
+  p.tiles_per_unit = 8.0 * cost(few) <= 7.0 * cost(run) ? few : run;
   p.units_per_cell = (ntiles + p.tiles_per_unit - 1) / p.tiles_per_unit;
   const int64_t units = (int64_t)p.n_cells * p.units_per_cell;
   const int grid = (int)std::min<int64_t>(units, sms);
-  fe_tc5_kernel<N, F16><<<grid, G::NT, G::BYTES, s>>>(p);
+  kernel<<<grid, G::NT, G::BYTES, s>>>(p);
   return cudaGetLastError();
 }
 
