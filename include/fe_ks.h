@@ -155,8 +155,9 @@ fe_ks_status fe_ks_quadrature_points(const fe_ks_problem* prob, double* xq_out);
  * coefficients (Sec. 3.1 eq. reformcellmat with the Jacobian scaling folded
  * in), cell-level projector matrices F^(a,e) (eq. Vnonloc), a conflict-free
  * colouring of the cells for the scatter-add, the GLL-lumped mass D, and all
- * device workspace for n_v_max vectors (up to 256 MiB of it assembly slots, one
- * per cell node on a shared DoF and column).  terms_mask selects the terms of H.
+ * device workspace for n_v_max vectors (assembly slots among it, one per cell
+ * node on a shared DoF and column, up to 256 MiB for FP64 storage and as much for
+ * FP32 storage).  terms_mask selects the terms of H.
  * cuda_stream (cudaStream_t, may be NULL = legacy default stream) orders all
  * later calls.  Returns FE_KS_ERR_MESH for out-of-range DoFs or det J <= 0.
  */
@@ -167,6 +168,14 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
  * Y = H X for n_v vectors (eq. HX).  X, Y: device [m][n_v] (complex:
  * interleaved) in the precision's storage type (double or float).  Y is
  * overwritten.  X and Y must not overlap.  1 <= n_v <= n_v_max.
+ *
+ * Applications of one context that may overlap on the device (fe_ks_set_stream,
+ * replayed graphs, a batch that names the context twice): an operator with
+ * projectors keeps its projections and assembly slots per storage width, so an
+ * application in FP64 storage (FE_KS_F64, FE_KS_F64E) may run beside one in FP32
+ * storage (the other precisions), while two of the same width must be ordered by
+ * the caller.  An operator without projectors has no such scratch: applications
+ * outside the set-up stream, or captured, take no slots and may all overlap.
  */
 fe_ks_status fe_ks_apply(fe_ks_ctx* ctx, const void* X, void* Y, int64_t n_v, int precision);
 

@@ -182,7 +182,7 @@ int greedy_colouring(int64_t E, int np3, int64_t m, const int* cell_dofs, int* c
 }
 
 // Most device memory a context sets aside for the slots of the one-launch
-// assembly.  Larger applications go colour by colour, where a colour's cells
+// assembly, per storage width.  Larger applications go colour by colour, where a colour's cells
 // then fill the device several times over and the launches cost nothing.
 constexpr size_t kAsmBytes = (size_t)256 << 20;
 
@@ -660,9 +660,13 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
   if (ok && !asm_dst.empty()) {
     // slots for as many columns as kAsmBytes holds (all of n_v_max where that is less); a
     // device too full for them goes colour by colour
-    const size_t full = (size_t)c->n_wslots * n_v_max * (c->cplx ? 2 : 1) * sizeof(double);
-    c->asm_bytes = std::min(full, kAsmBytes);
-    if (!(chk(upload<char>(c, reinterpret_cast<char**>(&c->asm_W), nullptr, c->asm_bytes)) &&
+    auto slots = [&](auto& od) {
+      const size_t column = (size_t)c->n_wslots * sizeof(*od.W);
+      od.slot_cols = n_v_max * (c->cplx ? 2 : 1);
+      if (column > 0) od.slot_cols = std::min<int64_t>(od.slot_cols, kAsmBytes / column);
+      return upload(c, &od.W, static_cast<decltype(od.W)>(nullptr), (size_t)c->n_wslots * od.slot_cols);
+    };
+    if (!(chk(slots(c->f64)) && chk(slots(c->f32)) &&
           chk(upload(c, &c->asm_dof, asm_dof.data(), asm_dof.size())) &&
           chk(upload(c, &c->asm_ptr, asm_ptr.data(), asm_ptr.size())) &&
           chk(upload(c, &c->asm_dst, asm_dst.data(), asm_dst.size())))) {
@@ -757,8 +761,8 @@ namespace feks {
 
 // Whether this application may go through the context's slots: the default kernel (cfg 0) or a
 // tensor-core one, slots large enough, and nobody else in them.  An operator with projectors
-// has per-context scratch anyway (Q and its partials), so its applications are ordered by the
-// caller; one without has none, and may run on several streams at once: only its set-up
+// has scratch of the same storage width anyway (Q and its partials), so its applications in that
+// width are ordered by the caller; one without has none, and may run on several streams at once: only its set-up
 // stream, and no graph captured there, takes the slots, every other application goes colour
 // by colour.  Tensor-core kernels, by colour -> one launch: FP16 p = 6, 8^3 cells, 64 columns
 // 288 -> 173 us; FP16 p = 3, 12^3, 16 columns 144 -> 91 us; BF16x2 p = 8, 8^3, 64 columns
@@ -785,7 +789,7 @@ static cudaError_t launch_cells(const Ctx& c, LocalParams<T, TS>& lp, bool one, 
     lp.cells = nullptr;
     lp.n_cells = (int)c.E;
     lp.dst = c.asm_dst;
-    lp.W = static_cast<TS*>(c.asm_W);
+    lp.W = asm_slots<TS>(c);
     lp.accum = accum;
     std::lock_guard<std::mutex> lk(c.asm_mu);   // another thread's pair of launches does not come between
     err = launch();

@@ -39,7 +39,7 @@ template <typename T, typename TV, int V>
 static cudaError_t assemble_v(const Ctx& c, T* Y, int64_t ncols, int accum, cudaStream_t s) {
   const int64_t total = c.n_shared * (ncols / V);
   const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)std::max(c.sms, 1) * 32);
-  fe_assemble_kernel<T, TV, V><<<blocks, 256, 0, s>>>(static_cast<const T*>(c.asm_W), Y, ncols, c.asm_dof, c.asm_ptr,
+  fe_assemble_kernel<T, TV, V><<<blocks, 256, 0, s>>>(asm_slots<T>(c), Y, ncols, c.asm_dof, c.asm_ptr,
                                                      total, (int)(ncols / V), accum);
   return cudaGetLastError();
 }

@@ -328,7 +328,7 @@ static fe_ks_status batch_build(fe_ks_batch* b) {
     d.np3 = c.np3;
     const bool slots = batch_slots(c, d.ncols, b->prec[s]);
     d.dst = slots ? c.asm_dst : nullptr;
-    d.W = c.asm_W;
+    d.W = f64 ? (void*)c.f64.W : (void*)c.f32.W;
     d.asm_dof = c.asm_dof;
     d.asm_ptr = c.asm_ptr;
     build_eo_tables<double>(c.p, c.nq, &P.t64[c.p]);

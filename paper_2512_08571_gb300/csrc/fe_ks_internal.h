@@ -52,6 +52,8 @@ struct OpData {
   T* dscale = nullptr;     // [m] D^{-1/2}
   T* Q = nullptr;          // workspace [n_atoms][n_proj][ncols_max]
   T* part = nullptr;       // projection partials [n_pairs][n_proj][ncols_max]
+  T* W = nullptr;          // assembly slots [n_wslots][columns], for up to slot_cols columns
+  int64_t slot_cols = 0;
   EOTables<T> tab;
 };
 
@@ -162,14 +164,13 @@ struct Ctx {
   float* cell_coef = nullptr;
   double gauss_w[kMaxN] = {};
   // one-launch assembly: destination of every cell node (row of Y when one cell
-  // meets the DoF, else ~slot of W), the shared DoFs with their slot ranges, and
-  // the slots' values
+  // meets the DoF, else ~slot) and the shared DoFs with their slot ranges.  The slots' values
+  // are per storage width (OpData::W), as Q and part are: applications of one context in FP64 and in
+  // FP32 storage may overlap
   int* asm_dst = nullptr;
   int* asm_dof = nullptr;
   int* asm_ptr = nullptr;    // [n_shared + 1]
   int64_t n_shared = 0, n_wslots = 0;
-  void* asm_W = nullptr;
-  size_t asm_bytes = 0;
   cudaStream_t home_stream = nullptr;   // of setup: the stream whose applications own the slots
   mutable std::mutex asm_mu;
   std::vector<void*> allocations;
@@ -246,7 +247,15 @@ template <typename T>
 cudaError_t launch_assemble(const Ctx& c, T* Y, int64_t ncols, int accum, cudaStream_t s);
 // whether one application of ncols columns of the given storage size fits the slots
 inline bool asm_fits(const Ctx& c, int64_t ncols, size_t esize) {
-  return c.asm_dst && (size_t)c.n_wslots * (size_t)ncols * esize <= c.asm_bytes;
+  return c.asm_dst && ncols <= (esize == 8 ? c.f64.slot_cols : c.f32.slot_cols);
+}
+// the slots' values in storage type T
+template <typename T>
+inline T* asm_slots(const Ctx& c) {
+  if constexpr (sizeof(T) == 8)
+    return c.f64.W;
+  else
+    return c.f32.W;
 }
 
 // kernel launchers (fe_ks_local_pN.cu)

@@ -320,3 +320,45 @@ def test_direct_systems_in_cuda_graph(batch_setup):
             _check(Ys, refs)
     finally:
         fk.fe_ks_batch_set_direct(b, None)
+
+
+@pytest.mark.parametrize("direct,split", [(None, (0, 0)), (None, (256, 384)), ([1, 1, 1, 1], (0, 0)),
+                                          ([1, 0, 0, 1], (0, 0)), ([0, 1, 1, 0], (256, 384))])
+def test_one_context_in_both_storage_widths(direct, split):
+    """Two contexts with projectors, each named as an FP64 and as an FP32 system of one batch: the four
+    systems overlap, so nothing they write may be shared between the widths (projections and assembly
+    slots).  Repeated; direct systems equal their own application bit for bit."""
+    stream = torch.cuda.current_stream().cuda_stream
+    wls = [Workload(f"w{s}", L=9.0, n=n, p=p, nq=p + 1, n_v=nv, gga=True, n_atoms=3, seed=7600 + s)
+           for s, (p, n, nv) in enumerate([(6, 4, 24), (5, 4, 40)])]
+    hps = [HostProblem(wl) for wl in wls]
+    ctxs = [fk.fe_ks_setup(hp.struct, fk.TERM_ALL, wl.n_v, stream) for hp, wl in zip(hps, wls)]
+    prec = [fk.FE_KS_F64, fk.FE_KS_F32, fk.FE_KS_F32, fk.FE_KS_F64]
+    own = [0, 0, 1, 1]
+    b = None
+    try:
+        Xs, refs = [], []
+        for s, pr in enumerate(prec):
+            X = torch.from_numpy(trial_vectors(wls[own[s]], seed_purpose=20 + s)).cuda().to(torch_dtype(pr, False))
+            R = torch.empty_like(X)
+            fk.fe_ks_apply(ctxs[own[s]], X, R, wls[own[s]].n_v, pr)
+            Xs.append(X)
+            refs.append(R)
+        b = fk.fe_ks_batch_create([ctxs[o] for o in own], [wls[o].n_v for o in own], prec)
+        fk.fe_ks_batch_set_split(b, *split)
+        fk.fe_ks_batch_set_direct(b, direct)
+        for _ in range(10):
+            Ys = [torch.full_like(X, float("nan")) for X in Xs]
+            fk.fe_ks_batch_apply(b, Xs, Ys, stream)
+            fk.fe_ks_batch_status(b)
+            for s, (Y, R) in enumerate(zip(Ys, refs)):
+                if direct and direct[s]:
+                    assert torch.equal(Y, R), s
+                else:
+                    err = parity_err(Y.double().cpu().numpy(), R.double().cpu().numpy())
+                    assert err <= TOL[prec[s]], (s, err)
+    finally:
+        if b is not None:
+            fk.fe_ks_batch_destroy(b)
+        for c in ctxs:
+            fk.fe_ks_destroy(c)

@@ -9,6 +9,7 @@ at the sizes where their tiles, column forms and assembly can go wrong.
 * The one-launch assembly gives the same bits twice, in every precision, and the bits of the
   colour-by-colour scatter (which a stream other than the set-up one takes for an operator
   without projectors).
+* Applications of one context in both storage widths may overlap.
 
 Tolerances as in test_parity_apply: 1e-12 for FP64 and pairs of floats, 1e-5 for FP32, per
 column and per entry.
@@ -132,6 +133,46 @@ def test_one_launch_gives_the_bits_of_the_colour_launches(precision, p, cplx, nv
         fk.fe_ks_destroy(ctx)
     assert not torch.isnan(ys[0]).any()
     assert torch.equal(ys[0], ys[1]) and torch.equal(ys[0], ys[2])
+
+
+@pytest.mark.parametrize("wide,narrow", [(fk.FE_KS_F64, fk.FE_KS_F32), (fk.FE_KS_F64E, fk.FE_KS_BF16)])
+def test_storage_widths_of_one_context_overlap(wide, narrow):
+    """An operator with projectors applied in FP64 and in FP32 storage on two streams, the FP32 ones
+    as replays of a captured graph: the bits of applications one after the other."""
+    wl = _wl(6, False, 0.05, n=4, n_v=40)
+    hp = HostProblem(wl)
+    X = torch.from_numpy(trial_vectors(wl)).cuda()
+    X32 = X.float()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    ctx = fk.fe_ks_setup(hp.struct, fk.TERM_ALL, wl.n_v, a.cuda_stream)
+    try:
+        ref, ref32 = torch.empty_like(X), torch.empty_like(X32)
+        torch.cuda.synchronize()
+        fk.fe_ks_apply(ctx, X, ref, wl.n_v, wide)
+        fk.fe_ks_apply(ctx, X32, ref32, wl.n_v, narrow)
+        torch.cuda.synchronize()
+        y32 = torch.empty_like(X32)
+        fk.fe_ks_set_stream(ctx, b.cuda_stream)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.stream(b):
+            graph.capture_begin()
+            for _ in range(4):
+                fk.fe_ks_apply(ctx, X32, y32, wl.n_v, narrow)
+            graph.capture_end()
+        fk.fe_ks_set_stream(ctx, a.cuda_stream)
+        ys = [torch.full_like(X, float("nan")) for _ in range(8)]
+        for _ in range(5):
+            y32.fill_(float("nan"))
+            torch.cuda.synchronize()
+            with torch.cuda.stream(b):
+                graph.replay()
+            for y in ys:
+                fk.fe_ks_apply(ctx, X, y, wl.n_v, wide)
+            torch.cuda.synchronize()
+            assert torch.equal(y32, ref32)
+            assert all(torch.equal(y, ref) for y in ys)
+    finally:
+        fk.fe_ks_destroy(ctx)
 
 
 @pytest.mark.parametrize("cplx", [False, True])
