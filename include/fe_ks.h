@@ -321,6 +321,15 @@ fe_ks_status fe_ks_device_status(fe_ks_ctx* ctx, int* status);
 fe_ks_status fe_ks_inject_fault(fe_ks_ctx* ctx, int kind);
 
 /*
+ * Host-side fault injection for tests into the calling thread's later
+ * fe_ks_setup calls, which succeed all the same: kind = 1 sets up contexts
+ * without assembly slots; kind = 2 makes the last of the slots' device
+ * allocations fail, as on a full device.  Either way every application goes
+ * colour by colour.  kind = 0 turns it off; FE_KS_ERR_ARG for another kind.
+ */
+fe_ks_status fe_ks_inject_setup_fault(int kind);
+
+/*
  * Cell-matrix (CM) baseline: the method the paper's matrix-free algorithms
  * are measured against (Sec. 3, eq. HX with precomputed H^(e)).  Real
  * operators only.

@@ -185,6 +185,7 @@ int greedy_colouring(int64_t E, int np3, int64_t m, const int* cell_dofs, int* c
 // assembly, per storage width.  Larger applications go colour by colour, where a colour's cells
 // then fill the device several times over and the launches cost nothing.
 constexpr size_t kAsmBytes = (size_t)256 << 20;
+static thread_local int g_setup_fault = 0;   // fe_ks_inject_setup_fault
 
 // ---- tile-configuration cache: fe_ks_tune's choice per (degree, n_q,
 // precision, columns, complex, device), reused by contexts of the same shape
@@ -657,20 +658,26 @@ fe_ks_status fe_ks_setup(const fe_ks_problem* prob, int terms_mask, int64_t n_v_
       }
     }
   }
-  if (ok && !asm_dst.empty()) {
+  if (ok && !asm_dst.empty() && g_setup_fault != 1) {
     // slots for as many columns as kAsmBytes holds (all of n_v_max where that is less); a
-    // device too full for them goes colour by colour
+    // device too full for them goes colour by colour, and keeps none of it
+    const size_t first = c->allocations.size();
     auto slots = [&](auto& od) {
       const size_t column = (size_t)c->n_wslots * sizeof(*od.W);
       od.slot_cols = n_v_max * (c->cplx ? 2 : 1);
       if (column > 0) od.slot_cols = std::min<int64_t>(od.slot_cols, kAsmBytes / column);
       return upload(c, &od.W, static_cast<decltype(od.W)>(nullptr), (size_t)c->n_wslots * od.slot_cols);
     };
-    if (!(chk(slots(c->f64)) && chk(slots(c->f32)) &&
-          chk(upload(c, &c->asm_dof, asm_dof.data(), asm_dof.size())) &&
+    if (!(chk(upload(c, &c->asm_dof, asm_dof.data(), asm_dof.size())) &&
           chk(upload(c, &c->asm_ptr, asm_ptr.data(), asm_ptr.size())) &&
-          chk(upload(c, &c->asm_dst, asm_dst.data(), asm_dst.size())))) {
-      c->asm_dst = nullptr;
+          chk(upload(c, &c->asm_dst, asm_dst.data(), asm_dst.size())) && chk(slots(c->f64)) &&
+          g_setup_fault != 2 && chk(slots(c->f32)))) {
+      for (size_t i = first; i < c->allocations.size(); ++i) cudaFree(c->allocations[i]);
+      c->allocations.resize(first);
+      c->asm_dof = c->asm_ptr = c->asm_dst = nullptr;
+      c->f64.W = nullptr;
+      c->f32.W = nullptr;
+      c->f64.slot_cols = c->f32.slot_cols = 0;
       g_last_error.clear();
     }
   }
@@ -1130,6 +1137,13 @@ fe_ks_status fe_ks_inject_fault(fe_ks_ctx* ctx, int kind) {
   if (!ctx) return fail(FE_KS_ERR_ARG, "ctx is NULL");
   if (kind != 0 && kind != 1) return fail(FE_KS_ERR_ARG, "kind must be 0 (off) or 1");
   ctx->c.inject_fault = kind;
+  return FE_KS_OK;
+}
+
+fe_ks_status fe_ks_inject_setup_fault(int kind) {
+  g_last_error.clear();
+  if (kind < 0 || kind > 2) return fail(FE_KS_ERR_ARG, "kind must be 0 (off), 1 or 2");
+  g_setup_fault = kind;
   return FE_KS_OK;
 }
 

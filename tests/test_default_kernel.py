@@ -175,6 +175,44 @@ def test_storage_widths_of_one_context_overlap(wide, narrow):
         fk.fe_ks_destroy(ctx)
 
 
+def test_set_up_on_a_full_device_keeps_no_slots():
+    """Set-up whose last slot allocation fails holds the memory of one without slots and gives the
+    same bits; one with slots holds at least their size more."""
+    wl = _wl(6, False, 0.05, n=6, n_v=64)
+    hp = HostProblem(wl)
+    X = torch.from_numpy(trial_vectors(wl)).cuda()
+    stream = torch.cuda.current_stream().cuda_stream
+    cells_per_dof = np.bincount(hp.dofs.ravel())
+    slots = int(cells_per_dof[cells_per_dof > 1].sum()) * wl.n_v * (8 + 4)
+    assert slots > 32 << 20
+    granule = 4 << 20                      # small allocations share device pages
+    try:
+        for _ in range(5):                 # the first set-up may load modules; others may use the device
+            ys, held = [], []
+            for kind in (0, 1, 2):
+                fk.fe_ks_inject_setup_fault(kind)
+                torch.cuda.synchronize()
+                free = torch.cuda.mem_get_info()[0]
+                ctx = fk.fe_ks_setup(hp.struct, fk.TERM_ALL, wl.n_v, stream)
+                try:
+                    held.append(free - torch.cuda.mem_get_info()[0])
+                    Y = torch.full_like(X, float("nan"))
+                    fk.fe_ks_apply(ctx, X, Y, wl.n_v, fk.FE_KS_F64)
+                    ys.append(Y)
+                    torch.cuda.synchronize()
+                finally:
+                    fk.fe_ks_destroy(ctx)
+            if abs(held[2] - held[1]) <= granule and held[0] - held[1] >= slots - granule:
+                break
+        else:
+            raise AssertionError(f"held {held}, slots {slots}")
+    finally:
+        fk.fe_ks_inject_setup_fault(0)
+    assert not torch.isnan(ys[0]).any() and all(torch.equal(ys[0], y) for y in ys)
+    with pytest.raises(fk.FeKsError, match="ERR_ARG"):
+        fk.fe_ks_inject_setup_fault(3)
+
+
 @pytest.mark.parametrize("cplx", [False, True])
 @pytest.mark.parametrize("precision", PREC)
 def test_projection_column_groups(precision, cplx):
