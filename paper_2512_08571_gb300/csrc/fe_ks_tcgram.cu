@@ -39,7 +39,7 @@
 // of 16), tcgen05.commit signals an mbarrier, all threads wait on it (bounded).
 //
 // What bounds it: instruction issue of the slicing (26 instructions a value) and of the
-// readout (47 an output), not the MMAs.  So everything else is taken off the chain: two
+// readout (53 an output), not the MMAs.  So everything else is taken off the chain: two
 // operand buffers, the next chunk sliced while this one's MMAs run and the one after
 // loaded to registers meanwhile, one block barrier per chunk, and the readout split so that the
 // warps that slice Z read fewer columns.  96 columns of 216000 rows: Gram 3.66 -> 0.68 ms, rotation
@@ -209,8 +209,8 @@ constexpr int NB0 = 5, NB1 = 3;   // blocks of 4 columns
 static_assert(2 * 4 * (NB0 + NB1) == TN, "readout split");
 
 // Read this thread's outputs of the chunk (row orow of the tile, nb blocks of 4 columns from
-// ocol0), combine the six accumulators in pairs of floats (the two smallest first, below 2^-28 of
-// the result; every other addition error-free), scale by 2^(E_row + E_col) and add to the running pairs.
+// ocol0), combine the six accumulators in pairs of floats (every addition error-free), scale by
+// 2^(E_row + E_col) and add to the running pairs.
 __device__ __forceinline__ void accumulate_chunk(uint32_t tmem, int warp, int orow, int ocol0, int nb, const int* Es,
                                                  float (&acc_hi)[4 * NB0], float (&acc_lo)[4 * NB0], int* sflag) {
   const int Ei = Es[orow];
@@ -226,10 +226,9 @@ __device__ __forceinline__ void accumulate_chunk(uint32_t tmem, int warp, int or
     for (int j = 0; j < 4; ++j) {
       const int jj = 4 * cb + j;
       const int E = Ei + Es[TILE + ocol0 + jj];
-      a[NACC - 2][j] += a[NACC - 1][j];
       float h = a[0][j], l = 0.f;
 #pragma unroll
-      for (int g = 1; g < NACC - 1; ++g) {
+      for (int g = 1; g < NACC; ++g) {
         float e;
         two_sum(h, a[g][j], h, e);
         l += e;

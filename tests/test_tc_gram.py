@@ -60,6 +60,29 @@ def test_tc_gram_of_a_general_product_on_its_upper_triangle():
     assert np.max(np.abs(C[iu] - ref[iu]) / scale[iu]) <= 1e-13
 
 
+def _two_level_chunk(s, t):
+    """32 values of two columns whose products are one of 1 by 0 and one of 0 by 1 (they set the
+    columns' exponents), 29 that fill the third 7-bit slice of both, and one of slices s and t."""
+    a, b = np.zeros(32), np.zeros(32)
+    a[0] = b[1] = 1.0
+    a[2:31] = b[2:31] = 127 * 2.0 ** -20
+    a[31], b[31] = 2.0 ** (-6 - 7 * s), 2.0 ** (-6 - 7 * t)
+    return a, b
+
+
+@pytest.mark.parametrize("s,t", [(2, 3), (3, 3), (3, 4), (0, 7)])
+def test_tc_products_add_the_last_accumulator_without_rounding(s, t):
+    """The fifth accumulator holds 29 * 127^2 and the sixth 1, 2^7 to 2^21 units further down: their sum
+    has 26 to 40 bits, more than an FP32 sum keeps, and is exact in a pair of floats and in FP64."""
+    a, b = _two_level_chunk(s, t)
+    want = 29 * 127 ** 2 * 2.0 ** -40 + 2.0 ** (-12 - 7 * (s + t))
+    Y = torch.from_numpy(np.stack([a, b], axis=1)).cuda()
+    C, status = fk.fe_ks_gram_tc_sym(Y, Y)
+    assert status == 0 and C[0, 1].item() == want and C[1, 0].item() == want
+    X, flags = fk.fe_ks_rotate_tc(torch.from_numpy(a[None].copy()).cuda(), torch.from_numpy(b[:, None].copy()).cuda())
+    assert flags == [0, 0] and X[0, 0].item() == want
+
+
 def test_tc_gram_zero_columns_and_out_of_range_scale():
     m, n = 9000, 40
     rng = np.random.default_rng(3)
