@@ -74,8 +74,17 @@ __global__ void k_rr_equilibrate(const double* __restrict__ S, double* __restric
 // rows in its lanes, so a step of the chain is a shuffle and an FMA, and what is not on the
 // chain spreads over the device.  One block doing a column at a time through global memory
 // took 461 us for the factor of a 96 x 96 matrix, one thread per right-hand side 430 us
-// for a solve; these take 178 and 28 us.
+// for a solve; these take 230 and 32 us.
 constexpr int kCb = 32;
+
+// x / d from r, 1 / d within an ulp or two: an FMA gives the residual of x r exactly, and r times it
+// corrects x r to the rounded quotient (P. Markstein, IBM J. Res. Dev. 34, 1990).  x r alone is a
+// rounding less accurate (a factor's error at n = 96 1.06 to 2.1 times) and takes 189 us a factor and
+// 27 a solve; x / d in place of this made a panel 105 instead of 88 us and a solve 55 instead of 38 (ncu).
+__device__ __forceinline__ double quotient(double x, double d, double r) {
+  const double q = x * r;
+  return fma(fma(-q, d, x), r, q);
+}
 
 // Panel of kCb columns at j0: every block factors the diagonal block (so none waits for
 // another), block b then solves the kCb rows below it that are its own, one row per lane.  The
@@ -87,7 +96,7 @@ __global__ void __launch_bounds__(kCb) k_rr_chol_panel(double* __restrict__ A, d
   __shared__ double Ls[kCb][kCb + 1];
   const int i = threadIdx.x, w = min(kCb, n - j0);
   if (__shfl_sync(0xffffffffu, *(volatile int*)flag, 0) != 0) return;
-  double row[kCb], rinv = 1.0;   // lane = row of the diagonal block (identity beyond w); 1 / L_ii
+  double row[kCb], rinv = 1.0;   // lane = row of the diagonal block (identity beyond w); about 1 / L_ii
 #pragma unroll
   for (int k = 0; k < kCb; ++k) row[k] = i < w && k < w && k <= i ? A[(int64_t)(j0 + i) * n + j0 + k] : (i == k ? 1.0 : 0.0);
 #pragma unroll
@@ -97,9 +106,9 @@ __global__ void __launch_bounds__(kCb) k_rr_chol_panel(double* __restrict__ A, d
       if (i == 0) *flag = 1 + j0 + j;
       return;
     }
-    const double ri = rsqrt(piv);
-    if (i == j) rinv = ri;
-    const double l = row[j] * ri;   // i == j: piv / sqrt(piv)
+    const double d = sqrt(piv), r = rsqrt(piv);
+    if (i == j) rinv = r;
+    const double l = i == j ? d : quotient(row[j], d, r);
     row[j] = l;
 #pragma unroll
     for (int k = j + 1; k < kCb; ++k) row[k] = fma(-l, __shfl_sync(0xffffffffu, l, k), row[k]);
@@ -116,7 +125,7 @@ __global__ void __launch_bounds__(kCb) k_rr_chol_panel(double* __restrict__ A, d
   for (int k = 0; k < kCb; ++k) x[k] = r < n ? A[(int64_t)r * n + j0 + k] : 0.0;
 #pragma unroll
   for (int k = 0; k < kCb; ++k) {
-    x[k] *= __shfl_sync(0xffffffffu, rinv, k);
+    x[k] = quotient(x[k], Ls[k][k], __shfl_sync(0xffffffffu, rinv, k));
 #pragma unroll
     for (int q = k + 1; q < kCb; ++q) x[q] = fma(-Ls[q][k], x[k], x[q]);
   }
@@ -196,11 +205,11 @@ __global__ void __launch_bounds__(128) k_rr_trsm(const double* __restrict__ L, d
       for (int k = 0; k < kCb; ++k) acc = fma(-Ls[lane][k], __shfl_sync(0xffffffffu, z, k), acc);
     }
     stage(ib, ib);
-    const double rinv = 1.0 / Ls[lane][lane];
+    const double d = Ls[lane][lane], rinv = 1.0 / d;
 #pragma unroll 8
     for (int q = 0; q < kCb; ++q) {
       const int j = TRANS ? kCb - 1 - q : q;
-      const double z = __shfl_sync(0xffffffffu, acc * rinv, j);
+      const double z = __shfl_sync(0xffffffffu, quotient(acc, d, rinv), j);
       if (lane == j) acc = z;
       if (TRANS ? lane < j : lane > j) acc = fma(-Ls[lane][j], z, acc);
     }
