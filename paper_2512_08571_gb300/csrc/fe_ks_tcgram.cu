@@ -39,11 +39,11 @@
 // of 16), tcgen05.commit signals an mbarrier, all threads wait on it (bounded).
 //
 // What bounds it: instruction issue of the slicing (26 instructions a value) and of the
-// readout (53 an output), not the MMAs.  So everything else is taken off the chain: two
+// readout (38 an output), not the MMAs.  So everything else is taken off the chain: two
 // operand buffers, the next chunk sliced while this one's MMAs run and the one after
 // loaded to registers meanwhile, one block barrier per chunk, and the readout split so that the
-// warps that slice Z read fewer columns.  96 columns of 216000 rows: Gram 3.66 -> 0.68 ms, rotation
-// 1.31 -> 0.74 ms.
+// warps that slice Z read fewer columns.  96 columns of 216000 rows: Gram 3.66 -> 0.64 ms, rotation
+// 1.31 -> 0.72 ms.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -209,8 +209,10 @@ constexpr int NB0 = 5, NB1 = 3;   // blocks of 4 columns
 static_assert(2 * 4 * (NB0 + NB1) == TN, "readout split");
 
 // Read this thread's outputs of the chunk (row orow of the tile, nb blocks of 4 columns from
-// ocol0), combine the six accumulators in pairs of floats (every addition error-free), scale by
-// 2^(E_row + E_col) and add to the running pairs.
+// ocol0), combine the six accumulators in pairs of floats, scale by 2^(E_row + E_col) and add to the
+// running pairs.  Every addition is error-free: the sum so far is a multiple of the units of the
+// accumulators in it, so of the last place of the next one, and for such terms the three operations
+// of Dekker's sum give the remainder whichever is larger.
 __device__ __forceinline__ void accumulate_chunk(uint32_t tmem, int warp, int orow, int ocol0, int nb, const int* Es,
                                                  float (&acc_hi)[4 * NB0], float (&acc_lo)[4 * NB0], int* sflag) {
   const int Ei = Es[orow];
@@ -229,9 +231,9 @@ __device__ __forceinline__ void accumulate_chunk(uint32_t tmem, int warp, int or
       float h = a[0][j], l = 0.f;
 #pragma unroll
       for (int g = 1; g < NACC; ++g) {
-        float e;
-        two_sum(h, a[g][j], h, e);
-        l += e;
+        const float s = h + a[g][j];
+        l += a[g][j] - (s - h);
+        h = s;
       }
       if (E < -126 || E > 127) {
         if (h != 0.f || l != 0.f) *sflag = 1;
