@@ -288,9 +288,12 @@ fe_ks_status fe_ks_cheb_filter_ghep(fe_ks_ctx* ctx, fe_ks_ctx* mass, double* X, 
  * this context and precision, and reports the milliseconds per call (-1 for
  * a configuration that cannot launch, e.g. shared memory too large) and the
  * choice. Y is overwritten. The choice also goes into an in-process cache
- * keyed by (degree, n_q, precision, columns, complex, device compute
- * capability and SM count). Other contexts of the same shape whose
- * configuration was not set explicitly use it at their next application.
+ * keyed by what the form of configuration 0 depends on: degree, n_q,
+ * precision, columns, complex, device compute capability and SM count, the
+ * cell count to a power of two, whether the assembly slots hold the columns
+ * and, for FE_KS_F32, whether every cell is an axis-aligned box. Other
+ * contexts of the same shape whose configuration was not set explicitly use it
+ * at their next application.
  *
  * fe_ks_set_config sets the configuration directly (and explicitly);
  * fe_ks_get_config reads the current one.

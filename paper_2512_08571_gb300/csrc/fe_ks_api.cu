@@ -188,22 +188,30 @@ constexpr size_t kAsmBytes = (size_t)256 << 20;
 static thread_local int g_setup_fault = 0;   // fe_ks_inject_setup_fault
 
 // ---- tile-configuration cache: fe_ks_tune's choice per (degree, n_q,
-// precision, columns, complex, device), reused by contexts of the same shape
-// whose configuration was not set explicitly.
+// precision, columns, complex, device, cells to a power of two, whether the
+// assembly slots hold the columns, whether FP32 cells are boxes), reused by
+// contexts of the same shape whose configuration was not set explicitly.  The
+// last three decide the form that configuration 0 takes: FP64, p = 4, 4^3 cells, 8
+// columns 24.6 us in one launch and 223 in the configurations by colour, one of
+// which is the fastest at 24^3 cells and 256 columns.
 namespace {
 struct TuneKey {
   int p, nq, prec, cplx, sm_major, sm_minor, sms;
   int64_t ncols;
+  int cells_log2, one, boxes;
   bool operator<(const TuneKey& o) const {
-    return std::tie(p, nq, prec, cplx, sm_major, sm_minor, sms, ncols) <
-           std::tie(o.p, o.nq, o.prec, o.cplx, o.sm_major, o.sm_minor, o.sms, o.ncols);
+    return std::tie(p, nq, prec, cplx, sm_major, sm_minor, sms, ncols, cells_log2, one, boxes) <
+           std::tie(o.p, o.nq, o.prec, o.cplx, o.sm_major, o.sm_minor, o.sms, o.ncols, o.cells_log2, o.one, o.boxes);
   }
 };
 std::mutex g_tune_mu;
 std::map<TuneKey, int> g_tune_cache;
 
 TuneKey tune_key(const Ctx& c, int prec, int64_t ncols) {
-  TuneKey k{c.p, c.nq, prec, c.cplx, 0, 0, 0, ncols};
+  TuneKey k{c.p, c.nq, prec, c.cplx, 0, 0, 0, ncols, 0, 0, 0};
+  for (int64_t e = c.E; e > 1; e >>= 1) ++k.cells_log2;
+  k.one = asm_fits(c, ncols, prec == FE_KS_F64 || prec == FE_KS_F64E ? 8 : 4);
+  k.boxes = prec == FE_KS_F32 && c.cell_coef != nullptr;
   cudaDeviceGetAttribute(&k.sm_major, cudaDevAttrComputeCapabilityMajor, c.device);
   cudaDeviceGetAttribute(&k.sm_minor, cudaDevAttrComputeCapabilityMinor, c.device);
   cudaDeviceGetAttribute(&k.sms, cudaDevAttrMultiProcessorCount, c.device);

@@ -6,7 +6,7 @@ import pytest
 
 from paper_2512_08571_gb300 import fe_ks as fk
 from synth.host_problem import HostProblem
-from synth import CONFIGS, trial_vectors
+from synth import CONFIGS, Workload, trial_vectors
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -36,4 +36,38 @@ def test_tuned_configuration_is_shared_by_same_shape_contexts():
         assert float(d.max()) < 1e-5
     finally:
         for ctx in (a, b, c):
+            fk.fe_ks_destroy(ctx)
+
+
+def test_tuned_configuration_stays_with_its_size_and_assembly():
+    """A choice made by colour (a context without assembly slots, where the pairs of floats at p = 6 prefer
+    another configuration than the default) reaches a context of the same mesh without slots, and none
+    with slots or with an eighth of the cells, whose default takes another form."""
+    p, n_v, prec = 6, 64, fk.FE_KS_F64E
+    big, small = (Workload("t", L=2.0 * n, n=n, p=p, nq=p + 1, n_v=n_v, gga=True, n_atoms=2, jitter=0.05, seed=99)
+                  for n in (8, 4))
+    hb, hs = HostProblem(big), HostProblem(small)
+    st = torch.cuda.current_stream().cuda_stream
+    X, Xs = torch.from_numpy(trial_vectors(big)).cuda(), torch.from_numpy(trial_vectors(small)).cuda()
+    ctxs = []
+
+    def setup(hp, kind):
+        fk.fe_ks_inject_setup_fault(kind)
+        try:
+            ctxs.append(fk.fe_ks_setup(hp.struct, fk.TERM_ALL, n_v, st))
+        finally:
+            fk.fe_ks_inject_setup_fault(0)
+        return ctxs[-1]
+
+    try:
+        best, ms = fk.fe_ks_tune(setup(hb, 1), X, torch.empty_like(X), n_v, prec, reps=5)
+        if best == 0:
+            pytest.skip("the tuner took the default")
+        for hp, kind, x, want in ((hb, 1, X, best), (hb, 0, X, 0), (hs, 1, Xs, 0)):
+            ctx = setup(hp, kind)
+            fk.fe_ks_apply(ctx, x, torch.empty_like(x), n_v, prec)
+            assert fk.fe_ks_get_config(ctx, prec) == want, (kind, x.shape)
+        torch.cuda.synchronize()
+    finally:
+        for ctx in ctxs:
             fk.fe_ks_destroy(ctx)
