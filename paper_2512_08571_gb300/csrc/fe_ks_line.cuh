@@ -190,12 +190,12 @@ enum : int { kLineFlat = 0, kLineWide = 1, kLineSmall = 2 };
 
 // Whether tiles of two elements give the fullest multiprocessor clearly (an eighth) less to do
 // than full ones: 64 cells of 8 FP64 columns at p = 4 took 31.8 us on 64 full tiles, 24.6 us on 256
-// of these; once every multiprocessor has several tiles the full ones' vector width wins
-template <int NQ>
+// of these; once every multiprocessor has several tiles the full ones' vector width wins.  VG, VS:
+// elements of a full and of a small tile; M: small ones are taken up to M eighths of the full ones' work
+template <int VG, int VS, int M = 7>
 bool line_small(int64_t slots, int sms) {
-  constexpr int VG = line_vg(NQ, false), VS = line_vg(NQ, true);
   const int64_t full = ((slots + VG - 1) / VG + sms - 1) / sms * VG, small = ((slots + VS - 1) / VS + sms - 1) / sms * VS;
-  return 8 * small <= 7 * full;
+  return 8 * small <= M * full;
 }
 
 // Shared memory of the wide form after the three tiles: [coefficients] [DoFs] [destinations] [a pair's
@@ -648,7 +648,8 @@ cudaError_t launch_line_t(const Ctx& c, const LocalParams<T, TS>& prm, cudaStrea
     for (size_t i = 0; i < sizeof(prm.tab) / 4; ++i) dst[i].v = (uint64_t)src[i] << 32 | src[i];
   }
   if constexpr (line_vg(NQ, true) < line_vg(NQ, false))
-    if (line_small<NQ>(elems, sms)) return launch_line_form<T, TS, NP, NQ, CPLX, BOX, kLineSmall>(c, lp, (elems + 1) / 2, sms, s);
+    if (line_small<line_vg(NQ, false), line_vg(NQ, true)>(elems, sms))
+      return launch_line_form<T, TS, NP, NQ, CPLX, BOX, kLineSmall>(c, lp, (elems + 1) / 2, sms, s);
   if constexpr (std::is_same<T, float>::value && NQ <= 9) {
     // wide form from one full tile of columns on; a unit's start (tables, first rows of X) costs about half a tile
     const int ntile = (ncg + S::VG - 1) / S::VG;

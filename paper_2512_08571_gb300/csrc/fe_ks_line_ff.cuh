@@ -63,6 +63,14 @@ struct LineShapeFF {
   static constexpr size_t bytes = 4 * (size_t)BUF * 8;
 };
 
+// line_small by the pairs' own widths.  At n_q = 7 a full tile has eight elements and two-element tiles
+// must save a quarter (p = 6, small / full: 512 slots 24.7 / 34.9 us, 2496 64.8 / 69.7; where they save
+// less: 3000 76 / 70, 5145 125 / 111).
+template <int NQ>
+bool line_ff_small(int64_t slots, int sms) {
+  return line_small<line_ff_vg(NQ, false), line_ff_vg(NQ, true), NQ == 7 ? 6 : 7>(slots, sms);
+}
+
 template <int NP, int NQ, bool CPLX, bool SMALL>
 __global__ void __launch_bounds__(LineShapeFF<NQ, SMALL>::NT, LineShapeFF<NQ, SMALL>::MINB)
     fe_line_ff_kernel(const __grid_constant__ LocalParams<ff2, double> p, int per_sm) {
@@ -268,7 +276,7 @@ cudaError_t launch_line_ff_t(const Ctx& c, const LocalParams<ff2, double>& prm, 
   const int sms = c.sms > 0 ? c.sms : 152;
   if (prm.n_cells == 0) return cudaSuccess;
   if constexpr (line_ff_vg(NQ, false) > 2)
-    if (line_small<NQ>((int64_t)prm.n_cells * prm.ncols, sms)) return launch_line_ff_form<NP, NQ, CPLX, true>(c, prm, sms, s);
+    if (line_ff_small<NQ>((int64_t)prm.n_cells * prm.ncols, sms)) return launch_line_ff_form<NP, NQ, CPLX, true>(c, prm, sms, s);
   return launch_line_ff_form<NP, NQ, CPLX, false>(c, prm, sms, s);
 }
 

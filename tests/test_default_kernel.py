@@ -62,9 +62,10 @@ def test_full_tiles(p, cplx, jitter):
     FP32, rows are not 8-byte aligned; the FP32 case runs the wide form (a block per cell)."""
     n = 3 if p < 3 else 2
     vg = 16 if p < 4 else 8 if p < 6 else 4
+    vgf = 8 if p == 6 else vg     # pairs of floats
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     elems = sms * vg // n ** 3 - 1
-    cols = {fk.FE_KS_F64: elems, fk.FE_KS_F64E: elems, fk.FE_KS_F32: 2 * elems - (0 if cplx else 1)}
+    cols = {fk.FE_KS_F64: elems, fk.FE_KS_F64E: sms * vgf // n ** 3 - 1, fk.FE_KS_F32: 2 * elems - (0 if cplx else 1)}
     nvs = {k: v // 2 if cplx else v for k, v in cols.items()}
     wl = _wl(p, cplx, jitter, n=n, n_v=max(nvs.values()))
     hp, X = HostProblem(wl), trial_vectors(wl)
