@@ -362,3 +362,47 @@ def test_one_context_in_both_storage_widths(direct, split):
             fk.fe_ks_batch_destroy(b)
         for c in ctxs:
             fk.fe_ks_destroy(c)
+
+
+@pytest.mark.parametrize("cells,depth,split", [(1, 1, (0, 0)), (3, 4, (0, 0)), (2, 2, (256, 384))])
+def test_colour_phases_beside_one_phase_systems(cells, depth, split):
+    """One queue of systems whose cells go in one phase (projectors and slots), by colour after the
+    projection phases (projectors, no slots) and by colour from phase 1 (no projectors), FP64 and FP32 of
+    each, for several claims a fetch and in split mode, against each system's own application."""
+    stream = torch.cuda.current_stream().cuda_stream
+    shapes = [  # degree, cells a side, columns, atoms, set up without slots (1)
+        (4, 3, 5, 2, 0), (5, 2, 9, 2, 1), (6, 3, 7, 0, 0), (8, 2, 6, 2, 0), (7, 2, 4, 2, 1), (4, 3, 12, 0, 0)]
+    precs = (fk.FE_KS_F64, fk.FE_KS_F32)
+    spec = [(*sh, precs[(s + k) % 2]) for k in (0, 1) for s, sh in enumerate(shapes)]
+    wls = [Workload(f"m{s}", L=3.0 * n, n=n, p=p, nq=p + 1, n_v=nv, gga=True, n_atoms=atoms, jitter=0.05, seed=7700 + s)
+           for s, (p, n, nv, atoms, _, _) in enumerate(spec)]
+    hps = [HostProblem(wl) for wl in wls]
+    ctxs, b = [], None
+    try:
+        for hp, wl, sp in zip(hps, wls, spec):
+            fk.fe_ks_inject_setup_fault(sp[4])
+            ctxs.append(fk.fe_ks_setup(hp.struct, fk.TERM_ALL, wl.n_v, stream))
+        fk.fe_ks_inject_setup_fault(0)
+        Xs, refs = [], []
+        for ctx, wl, sp in zip(ctxs, wls, spec):
+            X = torch.from_numpy(trial_vectors(wl)).cuda().to(torch_dtype(sp[5], False))
+            R = torch.empty_like(X)
+            fk.fe_ks_apply(ctx, X, R, wl.n_v, sp[5])
+            Xs.append(X)
+            refs.append(R)
+        b = fk.fe_ks_batch_create(ctxs, [wl.n_v for wl in wls], [sp[5] for sp in spec])
+        fk.fe_ks_batch_configure(b, [s % 2 for s in range(len(spec))], cells, depth, 2.0, False)
+        fk.fe_ks_batch_set_split(b, *split)
+        for _ in range(3):
+            Ys = [torch.full_like(X, float("nan")) for X in Xs]
+            fk.fe_ks_batch_apply(b, Xs, Ys, stream)
+            fk.fe_ks_batch_status(b)
+            for s, (Y, R) in enumerate(zip(Ys, refs)):
+                err = parity_err(Y.double().cpu().numpy(), R.double().cpu().numpy())
+                assert err <= TOL[spec[s][5]], (s, err)
+    finally:
+        fk.fe_ks_inject_setup_fault(0)
+        if b is not None:
+            fk.fe_ks_batch_destroy(b)
+        for c in ctxs:
+            fk.fe_ks_destroy(c)

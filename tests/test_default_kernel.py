@@ -9,6 +9,8 @@ at the sizes where their tiles, column forms and assembly can go wrong.
 * The one-launch assembly gives the same bits twice, in every precision, and the bits of the
   colour-by-colour scatter (which a stream other than the set-up one takes for an operator
   without projectors).
+* The same with projectors, in the small, flat and wide forms, and in the filter's accumulating
+  applications (contexts set up without slots go colour by colour).
 * Applications of one context in both storage widths may overlap.
 
 Tolerances as in test_parity_apply: 1e-12 for FP64 and pairs of floats, 1e-5 for FP32, per
@@ -174,6 +176,70 @@ def test_storage_widths_of_one_context_overlap(wide, narrow):
             assert all(torch.equal(y, ref) for y in ys)
     finally:
         fk.fe_ks_destroy(ctx)
+
+
+def _with_and_without_slots(hp, n_v, apply):
+    """[apply(ctx)] of a context with assembly slots and of one without, on the same operator."""
+    out = []
+    try:
+        for kind in (0, 1):
+            fk.fe_ks_inject_setup_fault(kind)
+            ctx = fk.fe_ks_setup(hp.struct, fk.TERM_ALL, n_v, torch.cuda.current_stream().cuda_stream)
+            try:
+                out.append(apply(ctx))
+                torch.cuda.synchronize()
+            finally:
+                fk.fe_ks_destroy(ctx)
+    finally:
+        fk.fe_ks_inject_setup_fault(0)
+    return out
+
+
+FORMS = [(5, 3, 3), (5, 4, 72), (8, 3, 40), (8, 3, 41)]   # p, cells a side, columns: small tiles, wide x 3
+
+
+@pytest.mark.parametrize("p,n,nv", FORMS)
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("precision", PREC + list(TC))
+def test_projectors_by_colour_and_in_one_launch(precision, cplx, p, n, nv):
+    """Operator with projectors: the expansion reaches the slots and the scatter by colour with the same
+    bits, in the small, flat and wide forms and in the tensor-core kernels, plain and scaled."""
+    hp = HostProblem(_wl(p, cplx, 0.05, n=n, n_v=nv))
+    X = torch.from_numpy(trial_vectors(_wl(p, cplx, 0.05, n=n, n_v=nv))).cuda().to(torch_dtype(precision, cplx))
+
+    def apply(ctx):
+        ys = [torch.full_like(X, float("nan")) for _ in range(2)]
+        fk.fe_ks_apply(ctx, X, ys[0], nv, precision)
+        fk.fe_ks_apply_scaled(ctx, X, ys[1], nv, precision)
+        return ys
+
+    one, colour = _with_and_without_slots(hp, nv, apply)
+    assert not any(torch.isnan(y).any() for y in one)
+    assert torch.equal(one[0], colour[0]) and torch.equal(one[1], colour[1])
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("precision", PREC + list(TC))
+def test_filter_by_colour_and_in_one_launch(precision, cplx):
+    """The filter's accumulating applications (Y += a H X) add to each row in the same order either way."""
+    p, n, nv = 8, 3, 40
+    wl = _wl(p, cplx, 0.05, n=n, n_v=nv)
+    hp = HostProblem(wl)
+    X = torch.from_numpy(trial_vectors(wl)).cuda()
+    ritz = torch.linspace(0.0, 5.0, nv, dtype=torch.float64, device="cuda")
+
+    def apply(ctx):
+        nb = fk.fe_ks_cheb_filter_workspace(ctx, nv, precision)
+        work = torch.empty(nb + 256, dtype=torch.uint8, device="cuda")
+        work = work[(-work.data_ptr()) % 256:][:nb]
+        y = X.clone()
+        fk.fe_ks_cheb_filter(ctx, y, ritz, nv, 5, 0.0, 10.0, 4000.0, precision, work, nb)
+        torch.cuda.synchronize()
+        return y
+
+    one, colour = _with_and_without_slots(hp, nv, apply)
+    assert torch.isfinite(torch.view_as_real(one) if cplx else one).all()
+    assert torch.equal(one, colour)
 
 
 def test_set_up_on_a_full_device_keeps_no_slots():
