@@ -65,7 +65,11 @@ typedef enum {
                                   their transposes) run on the tensor cores with BF16
                                   operands and FP32 accumulation, the quadrature-point terms,
                                   projections and scatter in FP32, the nonlocal expansion
-                                  as BF16 MMAs (apply / apply_scaled / tune / filter) */
+                                  as BF16 MMAs (apply / apply_scaled / tune / filter).
+                                  Slower than FE_KS_F32, as the other 16-bit precisions,
+                                  at every shape measured (p = 8, 256 columns, 24^3 cells
+                                  23.0 ms to 21.3, 12^3 3.4 to 3.0; p = 4, 10^3, 33
+                                  columns 125 us to 62): for 16-bit operands, not speed */
   FE_KS_F16 = 4,               /* as FE_KS_BF16 with FP16 operands (8x the precision): each
                                   column of a gathered cell tile is scaled by a power of two
                                   so that its largest entry is below 1/16, and unscaled at
@@ -157,7 +161,8 @@ fe_ks_status fe_ks_quadrature_points(const fe_ks_problem* prob, double* xq_out);
  * colouring of the cells for the scatter-add, the GLL-lumped mass D, and all
  * device workspace for n_v_max vectors (assembly slots among it, one per cell
  * node on a shared DoF and column, up to 256 MiB for FP64 storage and as much for
- * FP32 storage).  terms_mask selects the terms of H.
+ * FP32 storage, also where n_v_max columns need more: calls of fewer columns use
+ * them).  terms_mask selects the terms of H.
  * cuda_stream (cudaStream_t, may be NULL = legacy default stream) orders all
  * later calls.  Returns FE_KS_ERR_MESH for out-of-range DoFs or det J <= 0.
  */
@@ -405,7 +410,9 @@ fe_ks_status fe_ks_colour_cells(int64_t n_cells, int32_t np3, int64_t n_dofs, co
  * (re, im) columns, as for fe_ks_apply.
  * fe_ks_batch_configure sets the tunables -- tile configuration per system
  * (0/1: columns per tile), cells per work item, items claimed per fetch, resident CTAs per SM (1, or
- * 2 with a tighter register budget; 672-thread blocks run one per SM),
+ * 2 with a tighter register budget; 672-thread blocks run one per SM; until the first
+ * configure call a batch takes 2 where two CTAs of its systems fit an SM, else 1 -- eight small systems
+ * 870 us with 2, 1060 with 1 -- and a configure call, whatever else it sets, fixes the number it names),
  * threads per block (384, 512 or 672; 0 keeps the current, initially 384) --
  * plus the bounded-wait limit in seconds, and inject_missing_item = 1 makes
  * the host count one phase-0 item that is never published (fault injection:
@@ -443,9 +450,10 @@ fe_ks_status fe_ks_batch_set_split(fe_ks_batch* b, int threads_f64, int threads_
 /*
  * Direct systems: direct[s] != 0 (host array of n_sys flags; NULL clears all)
  * takes system s out of the persistent queue.  fe_ks_batch_apply then applies
- * it with its own context's kernels (projection and one tuned cell-kernel
- * launch per colour, as fe_ks_apply does, in the context's current tile
- * configuration), each direct system on a side stream of its own forked from
+ * it with its own context's kernels (as fe_ks_apply does, in the context's
+ * current tile configuration: the projection, then one cell-kernel launch and the sums of the
+ * shared rows for an operator with projectors whose slots hold the columns, else a launch per
+ * colour), each direct system on a side stream of its own forked from
  * cuda_stream with an event and joined back into it; the persistent launch of
  * the remaining systems (if any) runs on cuda_stream concurrently.  The whole
  * call still captures as one CUDA graph.  For a batch whose work is dominated
@@ -472,7 +480,8 @@ fe_ks_status fe_ks_info(const fe_ks_ctx* ctx, int64_t* n_dofs, int64_t* n_cells,
  * local kernels).  fe_ks_set_profiling(ctx, 1) starts recording (events are
  * created lazily, no device memory is allocated), 0 stops.
  * fe_ks_read_profile synchronises the recorded events and returns, for
- * phases 0 = zero-fill, 1 = nonlocal projection, 2 = fused local kernel, the
+ * phases 0 = zero-fill (none where all cells go in one launch), 1 = nonlocal
+ * projection, 2 = fused local kernel with the sums of the shared rows, the
  * total milliseconds ms[3] and the number of kernel launches launches[3] since
  * the last read, then clears them.
  */

@@ -968,10 +968,12 @@ cudaError_t launch_n(Params p, cudaStream_t s) {
   if (err != cudaSuccess) return err;
   const int ntiles = (p.ncols + G::VT - 1) / G::VT;
   // units of column tiles of one cell: even (the tiles alternate between the CTA's two pipelines),
-  // about 16 or more per SM, so that the cells with projectors, which take longer, spread; but the
+  // about 16 or more per SM, so that cells that take longer (those with projectors) spread; but the
   // run with the fewest rounds where that saves an eighth, a unit's start (coefficients, first gather
-  // and plane product, drained pipelines) costing about three tiles.  p = 8, 256 columns: 12^3 cells
-  // (216 a colour) 3.95 ms in 16 units per SM, 3.41 in the fewest rounds; 20^3, 32 atoms 13.7 and 14.4.
+  // and plane product, drained pipelines) costing about three tiles.  The rule goes by the counts alone.
+  // 256 columns, 16 units per SM / fewest rounds: p = 8, 12^3 cells (216 a colour) 3.95 / 3.41 ms; 20^3
+  // with 32 atoms 13.7 / 14.5, without 12.6 / 12.0; p = 6, 20^3 without 7.4 / 6.7; but p = 6, 3^3, 128
+  // columns without 29 / 30 us.
   int upc = 1;
   while (2 * upc < ntiles && (int64_t)p.n_cells * upc < 16LL * sms) upc *= 2;
   int run = (ntiles + upc - 1) / upc;

@@ -293,6 +293,8 @@ def fe_ks_batch_create(ctxs, n_v, precision):
 
 def fe_ks_batch_configure(batch, tile_config=None, cells_per_item=1, depth=1, wait_seconds=2.0,
                           inject_missing_item=False, blocks_per_sm=1, threads=0):
+    """Set every tunable.  blocks_per_sm (1 or 2) too: a batch takes 2 by itself where two blocks of its
+    systems fit a multiprocessor, but only until the first call here; name 2 to keep it."""
     tc = None if tile_config is None else (ctypes.c_int * len(tile_config))(*tile_config)
     _check(_lib.fe_ks_batch_configure(batch, tc, cells_per_item, depth, blocks_per_sm, wait_seconds,
                                       int(inject_missing_item), threads))
