@@ -330,7 +330,7 @@ __device__ __forceinline__ float tile_scale(float mx) {
 // when the rows are 16-byte aligned.  Colour-exclusive launches: no other
 // cell of the launch touches the same DoF rows.  One launch for all cells (dst):
 // plain stores to Y or to the node's slot.
-template <int N, bool CPLX, bool F16>
+template <int N, bool CPLX, bool F16, bool ONE>
 __device__ __forceinline__ void scatter_stage(const TcParams& p, const float* stage, const int* sd, int e, int c0,
                                               bool vecy, const float* unscale) {
   using Gm = Geom<N, CPLX>;
@@ -348,7 +348,7 @@ __device__ __forceinline__ void scatter_stage(const TcParams& p, const float* st
     const float sc = p.dscale ? p.alpha * __ldg(p.dscale + d) : p.alpha;
     a.x *= sc * ua.x, a.y *= sc * ua.y, a.z *= sc * ua.z, a.w *= sc * ua.w;
     b.x *= sc * ub.x, b.y *= sc * ub.y, b.z *= sc * ub.z, b.w *= sc * ub.w;
-    if (p.dst) {   // one launch for all cells: rows of one cell straight to Y, shared rows to their slots
+    if constexpr (ONE) {   // one launch for all cells: rows of one cell straight to Y, shared rows to their slots
       const int q = __ldg(p.dst + (int64_t)e * Gm::N3 + node);
       float* yp = q >= 0 ? p.Y + (int64_t)q * p.ld + c0 : p.W + (int64_t)(~q) * p.ld + c0;
       const bool add = p.accum && q >= 0;
@@ -382,8 +382,17 @@ __device__ __forceinline__ void scatter_stage(const TcParams& p, const float* st
   }
 }
 
-template <int N, bool CPLX, bool F16, bool SPLIT>
-__global__ void __launch_bounds__(Geom<N, CPLX, SPLIT>::NT, Geom<N, CPLX, SPLIT>::MINB)
+// Resident CTAs the registers are capped for.  One launch needs a few registers more than the launches
+// by colour, which sit at 96 in these two: 20 warps an SM, 16 above.
+template <int N, bool CPLX, bool F16, bool SPLIT, bool ONE>
+constexpr int min_blocks() {
+  return ONE && CPLX && !SPLIT && N == 6 ? 3 : ONE && CPLX && F16 && N == 4 ? 5 : Geom<N, CPLX, SPLIT>::MINB;
+}
+
+// ONE: one launch for all cells (p.dst), a variant of its own: as a run-time branch it cost the launches
+// by colour up to 16 % (complex, p = 5, FP16, 8^3 cells, 256 vectors 741 -> 860 us)
+template <int N, bool CPLX, bool F16, bool SPLIT, bool ONE>
+__global__ void __launch_bounds__(Geom<N, CPLX, SPLIT>::NT, (min_blocks<N, CPLX, F16, SPLIT, ONE>()))
     fe_tc_kernel(const __grid_constant__ TcParams p) {
   using Gm = Geom<N, CPLX, SPLIT>;
   constexpr bool K16 = Gm::K16;
@@ -428,7 +437,7 @@ __global__ void __launch_bounds__(Geom<N, CPLX, SPLIT>::NT, Geom<N, CPLX, SPLIT>
   const bool vecy = (p.ld % 4 == 0) && (((uintptr_t)p.Y & 15) == 0);
 
   for (int ci = blockIdx.x; ci < p.n_cells; ci += gridDim.x) {
-    const int e = p.cells ? p.cells[ci] : ci;
+    const int e = ONE ? ci : p.cells[ci];
     __syncthreads();   // the previous cell's scatter has finished with sd
     // stage the DoF list and the coefficients, point-major [pt][NC]
     for (int w = tid; w < N3; w += NT) sd[w] = p.cell_dofs[(int64_t)e * N3 + w];
@@ -480,7 +489,7 @@ __global__ void __launch_bounds__(Geom<N, CPLX, SPLIT>::NT, Geom<N, CPLX, SPLIT>
             if (p.dscale) sc[r] = __ldg(p.dscale + d);
           }
         }
-        if (prev0 >= 0) scatter_stage<N, CPLX, F16>(p, stage, sd, e, prev0, vecy, unscale);
+        if (prev0 >= 0) scatter_stage<N, CPLX, F16, ONE>(p, stage, sd, e, prev0, vecy, unscale);
         // FP16: scale every column of the tile by a power of two so that its
         // largest entry is below 1/16 (exact; undone at the scatter)
         float cs[8] = {1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f, 1.f};
@@ -863,7 +872,7 @@ __global__ void __launch_bounds__(Geom<N, CPLX, SPLIT>::NT, Geom<N, CPLX, SPLIT>
       __syncthreads();   // the stage is complete; array 2 is free for the next extraction
       prev0 = col0;
     }
-    if (prev0 >= 0) scatter_stage<N, CPLX, F16>(p, stage, sd, e, prev0, vecy, unscale);
+    if (prev0 >= 0) scatter_stage<N, CPLX, F16, ONE>(p, stage, sd, e, prev0, vecy, unscale);
   }
 }
 
@@ -874,12 +883,11 @@ cudaError_t launch_tc_n(const TcParams& p, cudaStream_t s) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaError_t err = cudaFuncSetAttribute(fe_tc_kernel<N, CPLX, F16, SPLIT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, Gm::BYTES);
+  auto kernel = p.dst ? fe_tc_kernel<N, CPLX, F16, SPLIT, true> : fe_tc_kernel<N, CPLX, F16, SPLIT, false>;
+  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Gm::BYTES);
   if (err != cudaSuccess) return err;
   // ask for the largest shared-memory carveout so that MINB CTAs fit on an SM with room to spare
-  err = cudaFuncSetAttribute(fe_tc_kernel<N, CPLX, F16, SPLIT>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
+  err = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (err != cudaSuccess) return err;
   const int ntiles = (p.ncols + 7) / 8;
   // about eight resident waves of CTAs: split the column tiles of a cell over
@@ -889,7 +897,7 @@ cudaError_t launch_tc_n(const TcParams& p, cudaStream_t s) {
   gy = gy < 1 ? 1 : (gy > ntiles ? ntiles : gy);
   if (gy > 65535) gy = 65535;
   const int gx = p.n_cells < (1 << 30) ? p.n_cells : (1 << 30);
-  fe_tc_kernel<N, CPLX, F16, SPLIT><<<dim3(gx, gy), Gm::NT, Gm::BYTES, s>>>(p);
+  kernel<<<dim3(gx, gy), Gm::NT, Gm::BYTES, s>>>(p);
   return cudaGetLastError();
 }
 
