@@ -34,6 +34,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <atomic>
+
 #include "fe_ks_internal.h"
 
 namespace feks {
@@ -894,6 +896,18 @@ cudaError_t launch_tc_n(const TcParams& p, cudaStream_t s) {
   // gridDim.y CTAs when the colour has few cells
   const int want = 8 * Gm::MINB * (sms > 0 ? sms : 152);
   int gy = (want + p.n_cells - 1) / p.n_cells;
+  if (p.dst) {
+    // one launch has no next colour to fill its last round: the units with the least time over the rounds
+    // of the CTAs that are resident, a unit's start (tables, an empty pipeline) costing about six tenths of a tile
+    static std::atomic<int> resident[64];
+    int r = resident[dev & 63].load(std::memory_order_relaxed);
+    if (r == 0) {
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, kernel, Gm::NT, Gm::BYTES) != cudaSuccess || r < 1) r = Gm::MINB;
+      resident[dev & 63].store(r, std::memory_order_relaxed);
+    }
+    const int run = tiles_per_unit(p.n_cells, ntiles, (int64_t)r * (sms > 0 ? sms : 152), 0.6);
+    gy = (ntiles + run - 1) / run;
+  }
   gy = gy < 1 ? 1 : (gy > ntiles ? ntiles : gy);
   if (gy > 65535) gy = 65535;
   const int gx = p.n_cells < (1 << 30) ? p.n_cells : (1 << 30);
