@@ -19,7 +19,8 @@ __global__ void __launch_bounds__(256) fe_assemble_kernel(const T* __restrict__ 
                                                           const int* __restrict__ dof, const int* __restrict__ ptr,
                                                           int64_t total, int groups, int accum) {
   for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < total; i += (int64_t)gridDim.x * 256) {
-    const int64_t s = i / groups;
+    // 32-bit division wherever the index fits (64-bit ones took most of a single column's time)
+    const int64_t s = i <= 0xFFFFFFFFll ? (int64_t)((uint32_t)i / (uint32_t)groups) : i / groups;
     const int64_t col = (i - s * groups) * V;
     const int b = ptr[s], e = ptr[s + 1];
     T* y = Y + (int64_t)dof[s] * ld + col;
@@ -48,6 +49,7 @@ template <>
 cudaError_t launch_assemble<float>(const Ctx& c, float* Y, int64_t ncols, int accum, cudaStream_t s) {
   if (c.n_shared == 0) return cudaSuccess;
   if (ncols % 4 == 0 && (uintptr_t)Y % 16 == 0) return assemble_v<float, float4, 4>(c, Y, ncols, accum, s);
+  if (ncols % 2 == 0 && (uintptr_t)Y % 8 == 0) return assemble_v<float, float2, 2>(c, Y, ncols, accum, s);
   return assemble_v<float, float, 1>(c, Y, ncols, accum, s);
 }
 template <>
