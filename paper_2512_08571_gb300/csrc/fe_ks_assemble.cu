@@ -19,7 +19,7 @@ __global__ void __launch_bounds__(256) fe_assemble_kernel(const T* __restrict__ 
                                                           const int* __restrict__ dof, const int* __restrict__ ptr,
                                                           int64_t total, int groups, int accum) {
   for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < total; i += (int64_t)gridDim.x * 256) {
-    // 32-bit division wherever the index fits (64-bit ones took most of a single column's time)
+    // 32-bit division wherever the index fits
     const int64_t s = i <= 0xFFFFFFFFll ? (int64_t)((uint32_t)i / (uint32_t)groups) : i / groups;
     const int64_t col = (i - s * groups) * V;
     const int b = ptr[s], e = ptr[s + 1];
