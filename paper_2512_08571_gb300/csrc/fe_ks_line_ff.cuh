@@ -51,7 +51,7 @@ __device__ __forceinline__ void eo_apply_ff(const ff2* x, const EOMat<ff2>& m, P
 constexpr int line_ff_vg(int nq, bool small) { return small ? 2 : nq >= 10 ? 2 : nq >= 8 ? 4 : nq >= 5 ? 8 : 16; }
 constexpr int line_ff_minb(int nq, bool small, int nt) {
   return small ? (768 / nt < 16 ? 768 / nt : 16)
-               : nq >= 11 ? 2 : nq == 10 ? 3 : nq == 9 ? 2 : nq == 8 ? 3 : nq == 7 ? 2 : nq == 6 ? 3 : nq == 5 ? 4 : 3;
+               : nq >= 11 ? 2 : nq == 10 ? 3 : nq == 9 ? 2 : nq == 8 ? 3 : nq == 7 ? 2 : nq == 6 ? 3 : nq == 5 ? 4 : nq == 4 ? 3 : nq == 3 ? 6 : 12;
 }
 template <int NQ, bool SMALL = false>
 struct LineShapeFF {
