@@ -276,7 +276,9 @@ fe_ks_status fe_ks_cheb_filter_ghep(fe_ks_ctx* ctx, fe_ks_ctx* mass, double* X, 
  *         shape: a block per cell with its tables in shared memory (FP32, a tile
  *         of columns or more), flattened tiles otherwise, small ones for small
  *         problems; all cells in one launch where the context's assembly slots
- *         hold the columns, else a launch per colour (same bits);
+ *         hold the columns, else a launch per colour (same bits).  FE_KS_F64E with large
+ *         blocks at n_q <= 6 (60 to 500 thousand cells times columns on) and n_q = 10 (real,
+ *         25 thousand): the kernel of 1..2 with its narrowest tile, a launch per colour;
  *   1..2  one CTA per (cell, column tile), 2 tile widths;
  *   3..4  one CTA per cell walking all column tiles, the next tile's rows of X
  *         staged by cp.async, reduction-based scatter;

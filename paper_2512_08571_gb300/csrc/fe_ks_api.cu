@@ -941,7 +941,7 @@ fe_ks_status apply_core_emu(Ctx& c, const double* X, double* Y, int64_t ncols, b
     c.ev_pool.pop_back();
     cudaEventRecord(ev[i], s);
   };
-  const bool one = one_launch(c, c.cfgE, ncols, sizeof(double));
+  const bool one = !ff_tiles(c, ncols) && one_launch(c, c.cfgE, ncols, sizeof(double));
   mark(0);
   if (zero_fill && !one && cudaMemsetAsync(Y, 0, bytes, s) != cudaSuccess)
     return fail(FE_KS_ERR_CUDA, "cudaMemsetAsync failed");

@@ -258,6 +258,24 @@ inline T* asm_slots(const Ctx& c) {
     return c.f32.W;
 }
 
+// Pairs of floats, tile configuration 0: whether an application of ncols columns runs the kernel of one CTA
+// per (cell, column tile) in fe_ks_local.cuh, by colour, instead of the line kernel.  The line kernel's rolled
+// loops and one launch win by up to 6 times on small blocks; on large ones of few points a line its
+// slots and run-time strides cost more than they save, and a real n_q = 10 has shared memory for 21 warps an SM
+// against 26.  Elements from which on the tile kernel is faster, line / tile kernel there and at the
+// largest measured: n_q = 2 at 512 thousand (p = 1, complex) 1.03, 767 1.14; 3 at 376 1.05, 767 1.14;
+// 4 at 376 1.04, 512 1.10; 5 at 188 1.02, 767 1.05; 6 at 64 1.06, 512 1.14; real 10 at 31 1.10 to 1.16.
+inline bool ff_tiles(const Ctx& c, int64_t ncols) {
+  const int64_t from = c.nq == 2   ? 500000
+                       : c.nq == 3 ? 300000
+                       : c.nq == 4 ? 280000
+                       : c.nq == 5 ? 160000
+                       : c.nq == 6 ? 60000
+                       : c.nq == 10 && !c.cplx ? 25000
+                                             : INT64_MAX;
+  return c.E * ncols >= from;
+}
+
 // kernel launchers (fe_ks_local_pN.cu)
 template <typename T, typename TS>
 cudaError_t launch_local(const Ctx& c, const LocalParams<T, TS>& prm, cudaStream_t s);

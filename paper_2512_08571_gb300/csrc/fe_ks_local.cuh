@@ -1176,7 +1176,10 @@ cudaError_t launch_local_deg(const Ctx& c, const LocalParams<T, TS>& prm, cudaSt
     case 7: return launch_lean_cfg<T, TS, NP, NQ, V1, cfg_nt(V1 / 2, NQ), 2, 2>(c, prm, s);
     case 8: return launch_lean_cfg<T, TS, NP, NQ, V1, cfg_nt(V1 / 4, NQ), 4, 2>(c, prm, s);
     case 9: return launch_lean_cfg<T, TS, NP, NQ, V0, cfg_nt(V0 / 2, NQ), 2, 3>(c, prm, s);
-    default: return launch_line_deg<T, TS, P, NQX>(c, prm, s);
+    default:
+      if constexpr (std::is_same<T, ff2>::value && (NQ <= 6 || NQ == 10))
+        if (!prm.dst && ff_tiles(c, prm.ncols)) return launch_local_cfg<T, TS, NP, NQ, V0, cfg_nt(V0, NQ)>(c, prm, s);
+      return launch_line_deg<T, TS, P, NQX>(c, prm, s);
   }
 }
 

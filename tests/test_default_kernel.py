@@ -242,6 +242,40 @@ def test_filter_by_colour_and_in_one_launch(precision, cplx):
     assert torch.equal(one, colour)
 
 
+@pytest.mark.parametrize("p,nqx,cplx,first", [(1, 0, False, 500000), (2, 0, True, 300000), (3, 0, False, 280000),
+                                              (1, 2, True, 280000), (4, 0, False, 160000), (2, 2, True, 160000),
+                                              (5, 0, True, 60000), (3, 2, False, 60000), (7, 2, False, 25000)])
+def test_large_blocks_in_pairs_of_floats(p, nqx, cplx, first):
+    """Blocks on both sides of the line from which the pairs of floats take the kernel by tiles and
+    colours: every column as a small block of the line kernel gives it, to rounding; the same bits twice
+    and with and without slots; the block below the line in one launch."""
+    n, cw = 4, 2 if cplx else 1
+    nv = -(-first // (n ** 3 * cw))
+    wl = _wl(p, cplx, 0.05, nqx=nqx, n=n, n_v=nv)
+    hp = HostProblem(wl)
+    X = torch.from_numpy(trial_vectors(wl)).cuda()
+    some = torch.tensor([0, 1, 2, nv // 2, nv - 3, nv - 2], device="cuda")
+
+    def apply(ctx):
+        out = []
+        for cols in (nv, nv, nv - 1, None):
+            x = X[:, some].contiguous() if cols is None else X[:, :cols].contiguous()
+            y = torch.full_like(x, float("nan"))
+            fk.fe_ks_set_profiling(ctx, 1)
+            fk.fe_ks_apply(ctx, x, y, x.shape[1], fk.FE_KS_F64E)
+            out.append((y, fk.fe_ks_read_profile(ctx)["fill"][1]))
+        return out
+
+    one, colour = _with_and_without_slots(hp, nv, apply)
+    (a, fa), (b, _), (below, fb), (small, _) = one
+    assert torch.equal(a, b) and torch.equal(a, colour[0][0])
+    assert (fa, fb) == (1, 0)                  # launches by colour start from a zero-fill, one launch does not
+    small = small.cpu().numpy()
+    for y in (a, below):
+        assert not torch.isnan(y).any()
+        assert parity_err(y[:, some].cpu().numpy(), small) <= TOL[fk.FE_KS_F64E]
+
+
 def test_set_up_on_a_full_device_keeps_no_slots():
     """Set-up whose last slot allocation fails holds the memory of one without slots and gives the
     same bits; one with slots holds at least their size more."""
