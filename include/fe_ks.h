@@ -413,8 +413,9 @@ fe_ks_status fe_ks_colour_cells(int64_t n_cells, int32_t np3, int64_t n_dofs, co
  * fe_ks_batch_configure sets the tunables -- tile configuration per system
  * (0/1: columns per tile), cells per work item, items claimed per fetch, resident CTAs per SM (1, or
  * 2 with a tighter register budget; 672-thread blocks run one per SM; until the first
- * configure call a batch takes 2 where two CTAs of its systems fit an SM, else 1 -- eight small systems
- * 870 us with 2, 1060 with 1 -- and a configure call, whatever else it sets, fixes the number it names),
+ * configure call a batch takes 2 where two CTAs of its systems fit an SM and the phases of no system are a
+ * chain of more than three times the work, else 1 -- eight small systems 870 us with 2, 1060 with 1 -- and
+ * a configure call, whatever else it sets, fixes the number it names),
  * threads per block (384, 512 or 672; 0 keeps the current, initially 384) --
  * plus the bounded-wait limit in seconds, and inject_missing_item = 1 makes
  * the host count one phase-0 item that is never published (fault injection:

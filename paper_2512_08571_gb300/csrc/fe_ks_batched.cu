@@ -113,7 +113,7 @@ struct fe_ks_batch {
   int cells_per_item = 1;
   int depth = 1;
   int blocks_per_sm = 0;     // 1: registers for every variant; 2: two CTAs per SM, some spills; 0 (until
-                             // configured): 2 where the systems' tiles let two share an SM, else 1
+                             // configured): by the rule in batch_build
   int bps = 1;               // the one in use
   int nt = kBatchThreads[0]; // threads per CTA (one of kBatchThreads)
   double wait_seconds = 2.0;
@@ -244,6 +244,27 @@ static fe_ks_status batch_build(fe_ks_batch* b) {
     for (auto& v : pp)
       std::stable_sort(v.begin(), v.end(), [&](const int4& a, const int4& c) { return cost(a) > cost(c); });
   };
+  // work of the cell items of a multiprocessor, and the longest system's phases one after the other when each
+  // phase spreads over the multiprocessors (a tile's columns that do not exist cost nothing)
+  double work = 0.0, chain = 0.0;
+  if (!split) {
+    std::vector<double> path(ns, 0.0);
+    for (const auto& v : per_phase) {
+      std::vector<double> item(ns, 0.0);
+      std::vector<int64_t> count(ns, 0);
+      for (const int4& w : v) {
+        const int s = w.x & 0xff, vt = vt_of(b->ctxs[s]->c.p, b->cfg[s]);
+        const double t = cost(w) * std::min<int64_t>(vt, b->n_v[s] - w.z) / vt;
+        if (t <= 0.0) continue;
+        work += t / b->sms;
+        item[s] += t;
+        ++count[s];
+      }
+      for (int s = 0; s < ns; ++s)
+        if (count[s]) path[s] += item[s] / count[s] * ((count[s] + b->sms - 1) / b->sms);
+    }
+    chain = *std::max_element(path.begin(), path.end());
+  }
   longest_first(per_phase);
   longest_first(per_phase_cls[0]);
   longest_first(per_phase_cls[1]);
@@ -282,8 +303,11 @@ static fe_ks_status batch_build(fe_ks_batch* b) {
     b->smem = std::max<size_t>(smem, 16);
     int per_sm = 0;
     // two blocks hide each other's barriers and FP64 latencies: eight small systems 1060 -> 870 us, twelve
-    // of up to 7^3 cells 4850 -> 4010 us, in spite of the spills
-    b->bps = b->blocks_per_sm ? b->blocks_per_sm : 2;
+    // of up to 7^3 cells 4850 -> 4010 us, in spite of the spills.  But where the phases of one system, by
+    // colour, are a chain of several times the work, a block to itself takes an item faster: an FP64 system
+    // of 4^3 cells, p = 8, 12 columns, without projectors beside two FP32 ones (chain 6 times the work) 770 us
+    // with one block, 926 with two; chain 4.6 times 1900 / 2058; up to 2 times within 2 % or two are faster
+    b->bps = b->blocks_per_sm ? b->blocks_per_sm : chain > 3.0 * work ? 1 : 2;
     cudaError_t perr = prepare_nt(b->nt, b->smem, b->bps, &per_sm);
     if (!b->blocks_per_sm && (perr != cudaSuccess || per_sm < 2)) {
       cudaGetLastError();

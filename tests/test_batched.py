@@ -406,3 +406,35 @@ def test_colour_phases_beside_one_phase_systems(cells, depth, split):
             fk.fe_ks_batch_destroy(b)
         for c in ctxs:
             fk.fe_ks_destroy(c)
+
+
+@pytest.mark.parametrize("atoms,blocks", [(0, 1), (2, 2)])
+def test_blocks_per_multiprocessor_of_a_fresh_batch(atoms, blocks):
+    """A fresh batch runs two blocks a multiprocessor, but one where a system's colour phases, each with
+    fewer items than multiprocessors, are a chain that outlasts the work; a configure call fixes the number."""
+    stream = torch.cuda.current_stream().cuda_stream
+    spec = [(8, 4, 12, fk.FE_KS_F64), (5, 2, 4, fk.FE_KS_F32)]
+    wls = [Workload(f"f{s}", L=3.0 * n, n=n, p=p, nq=p + 1, n_v=nv, gga=True, n_atoms=atoms, seed=7800 + s)
+           for s, (p, n, nv, _) in enumerate(spec)]
+    hps = [HostProblem(wl) for wl in wls]
+    ctxs = [fk.fe_ks_setup(hp.struct, fk.TERM_ALL, wl.n_v, stream) for hp, wl in zip(hps, wls)]
+    b = None
+    try:
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        b = fk.fe_ks_batch_create(ctxs, [wl.n_v for wl in wls], [sp[3] for sp in spec])
+        assert fk.fe_ks_batch_info(b)["grid"] == blocks * sms
+        Xs = [torch.from_numpy(trial_vectors(wl)).cuda().to(torch_dtype(sp[3], False)) for wl, sp in zip(wls, spec)]
+        Ys, refs = [torch.full_like(X, float("nan")) for X in Xs], [torch.empty_like(X) for X in Xs]
+        fk.fe_ks_batch_apply(b, Xs, Ys, stream)
+        fk.fe_ks_batch_status(b)
+        for ctx, X, Y, R, sp in zip(ctxs, Xs, Ys, refs, spec):
+            fk.fe_ks_apply(ctx, X, R, X.shape[1], sp[3])
+            assert parity_err(Y.double().cpu().numpy(), R.double().cpu().numpy()) <= TOL[sp[3]]
+        for occ in (1, 2):
+            fk.fe_ks_batch_configure(b, blocks_per_sm=occ)
+            assert fk.fe_ks_batch_info(b)["grid"] == occ * sms
+    finally:
+        if b is not None:
+            fk.fe_ks_batch_destroy(b)
+        for c in ctxs:
+            fk.fe_ks_destroy(c)
