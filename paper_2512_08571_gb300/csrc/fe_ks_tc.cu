@@ -896,9 +896,14 @@ cudaError_t launch_tc_n(const TcParams& p, cudaStream_t s) {
   // gridDim.y CTAs when the colour has few cells
   const int want = 8 * Gm::MINB * (sms > 0 ? sms : 152);
   int gy = (want + p.n_cells - 1) / p.n_cells;
-  if (p.dst) {
-    // one launch has no next colour to fill its last round: the units with the least time over the rounds
-    // of the CTAs that are resident, a unit's start (tables, an empty pipeline) costing about six tenths of a tile
+  gy = gy < 1 ? 1 : (gy > ntiles ? ntiles : gy);
+  if (N >= 6 && p.dst && ntiles >= 4 * gy) {
+    // one launch has no next colour to fill its last round, and units of four tiles or more can leave it nearly
+    // empty: the units with the least time over the rounds of the CTAs that are resident, a unit's start
+    // (tables, an empty pipeline) costing about six tenths of a tile.  Eight waves / these, split precision,
+    // 8^3 cells: p = 8, 152 columns 1511 / 1415 us, p = 7, 226 columns 1432 / 1331, p = 5, 250 columns 709 / 671.
+    // Smaller units and fewer points stay with eight waves: p = 7, 27 columns 118 / 127 us, p = 2, 16^3 cells,
+    // 512 columns in BF16 1146 / 1256.
     static std::atomic<int> resident[64];
     int r = resident[dev & 63].load(std::memory_order_relaxed);
     if (r == 0) {
@@ -908,7 +913,6 @@ cudaError_t launch_tc_n(const TcParams& p, cudaStream_t s) {
     const int run = tiles_per_unit(p.n_cells, ntiles, (int64_t)r * (sms > 0 ? sms : 152), 0.6);
     gy = (ntiles + run - 1) / run;
   }
-  gy = gy < 1 ? 1 : (gy > ntiles ? ntiles : gy);
   if (gy > 65535) gy = 65535;
   const int gx = p.n_cells < (1 << 30) ? p.n_cells : (1 << 30);
   kernel<<<dim3(gx, gy), Gm::NT, Gm::BYTES, s>>>(p);
